@@ -124,6 +124,7 @@ struct mg_ctx {
   // abandon, and the stall test (mg_ctx_set_wait_limit)
   unsigned long long wait_ns = 4000000000ull;
   int stall_test = 0;
+  int sms = 1;                // multiprocessors of the device
   // algorithmic work of predicated squaring launches, added on the device (timing on)
   double* dev_flops = nullptr;
   std::string tune_cache;   // tuning cache consulted by servers for MG_PREC_AUTO jobs
@@ -184,6 +185,7 @@ enum Slot {
   WS_ACT_REC,   // action path: interval records, off-chip interval matrices, send masks, job records
   WS_TRAJ,      // trajectory output staged on the device (host output buffers)
   WS_SEG_A, WS_SEG_B, WS_SEG_I,   // segmented tree: gathered operand pairs, their indices
+  WS_F64_SUMS,   // FP64 products from digits: per-CTA sums between the sweeps
   WS_COUNT
 };
 
@@ -352,6 +354,13 @@ int timing_mark(mg_ctx* ctx, int* idx) {
   return MG_OK;
 }
 
+// Smallest dimension whose FP64 products run from digits on the tensor cores.  Up to 32 the
+// FP64-pipe kernel covers a product with one 32 x 32 tile and is faster (exponentials of 512
+// matrices: d = 32 1.54 ms against 2.00 ms from digits); beyond, its 64 x 64 tiles pad the
+// FP64 work and the digits win at every batch (d = 40: 6.74 against 2.44 ms, one matrix 1.79
+// against 0.77 ms; d = 128: 79.9 against 7.7 ms).
+constexpr int kF64DigitsMinDim = 33;
+
 struct Engine {
   mg_ctx* ctx;
   int d, prec, L;
@@ -371,6 +380,9 @@ struct Engine {
   bool x_sym = false;                 // ... and symmetric: every polynomial in X is symmetric
   int a_zero = 0, b_zero = 0;         // structure of the next product's operands
   int sym = 0;                        // the next product's result is complex symmetric
+  bool fp64_pipe = false;             // FP64 products on the FP64 pipe at every dimension (mg_cgemm)
+  // FP64 products from integer digits on the tensor cores (gemm_f64_digits.cu)
+  bool digits64() const { return prec == MG_PREC_FP64 && !fp64_pipe && d >= kF64DigitsMinDim; }
   bool allow18() const { return prec == MG_PREC_SPLIT && taylor_mode != MG_TAYLOR_PS; }
   SplitCtl ctl() const {
     SplitCtl c;
@@ -388,6 +400,13 @@ struct Engine {
   }
 
   int reserve(int batch) {
+    if (digits64()) {
+      MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(d, batch), &abuf));
+      MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(d, batch), &bbuf[0]));
+      MG_TRY(ws_get(ctx, WS_BBUF1, f64d_b_bytes(d, batch), &bbuf[1]));
+      void* sums;
+      return ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms), &sums);
+    }
     if (prec != MG_PREC_SPLIT) return MG_OK;
     MG_TRY(ws_get(ctx, WS_ABUF, split_a_bytes(d, L, batch), &abuf));
     MG_TRY(ws_get(ctx, WS_BBUF0, split_b_bytes(d, L, batch), &bbuf[0]));
@@ -398,10 +417,12 @@ struct Engine {
   // the FP64 path stores FP64.  Both use 16 bytes per complex element.
   bool df() const { return prec == MG_PREC_SPLIT; }
   int prepA(int batch, const double* A, long long sA, int in_df) {
+    if (digits64()) return f64d_slice_a(d, batch, A, sA, 0, abuf, ctx->stream, ctl());
     if (prec != MG_PREC_SPLIT) return MG_OK;
     return split_slice_a(d, L, batch, A, sA, in_df, abuf, ctx->stream, ctl());
   }
   int prepB(int slot, int batch, const double* B, long long sB, int in_df) {
+    if (digits64()) return f64d_slice_b(d, batch, B, sB, bbuf[slot], ctx->stream, ctl());
     if (prec != MG_PREC_SPLIT) return MG_OK;
     return split_slice_b(d, L, batch, B, sB, in_df, bbuf[slot], ctx->stream, ctl());
   }
@@ -419,7 +440,7 @@ struct Engine {
   // skipping never read (the zero half of A's K axis; the zero plane of B, or both -Im
   // and Im planes of a real B).  Otherwise the general slicers.
   int prep_poly(bool as_a, int slot, int batch, const double* M, int part) {
-    if (prec != MG_PREC_SPLIT) return MG_OK;
+    if (prec != MG_PREC_SPLIT && !digits64()) return MG_OK;
     if (!lower()) {
       if (as_a) MG_TRY(prepA(batch, M, mat_doubles_(), 1));
       if (slot >= 0) MG_TRY(prepB(slot, batch, M, mat_doubles_(), 1));
@@ -466,7 +487,8 @@ struct Engine {
     return df() ? launch_fp64_to_df(batch, d, src, ss, dst, ds, ctx->stream)
                 : launch_copy_strided(batch, 2LL * d * d, src, ss, dst, ds, ctx->stream);
   }
-  // C = A B (+ addends); split mode uses the digits prepared by prepA / prepB(slot).
+  // C = A B (+ addends); split mode and FP64 from digits use the digits prepared by prepA /
+  // prepB(slot) (the latter reads A and B too, for items outside the digits' range).
   int mul(int batch, const double* A, long long sA, int slot, const double* B, long long sB, double* C,
           long long sC, const AddTerms& add) {
     products += batch;
@@ -481,6 +503,9 @@ struct Engine {
     if (prec == MG_PREC_SPLIT) {
       r = split_gemm(d, L, batch, abuf, bbuf[slot], C, sC, add, ctx->status, ctx->stream, ctl());
       a_zero = b_zero = sym = 0;
+    } else if (digits64()) {
+      r = f64d_gemm(d, batch, 0, A, sA, abuf, B, sB, bbuf[slot], C, sC, add, ctx->slot_ptr[WS_F64_SUMS], ctx->sms,
+                    ctx->status, ctx->stream, ctl());
     } else {
       AddTerms a = add;
       a.item_sq = item_sq;
@@ -732,7 +757,8 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
     for (int k = 0; k < S; ++k) {
       eng.item_sq = sq_dev;
       eng.sq_step = k;
-      int r = eng.mul(batch, R, md, 0, R, md, Rn, md, none);
+      int r = eng.prep_poly(true, 0, batch, R, 0);
+      if (r == MG_OK) r = eng.mul(batch, R, md, 0, R, md, Rn, md, none);
       if (r == MG_OK) r = launch_copy_active(batch, md, Rn, R, sq_dev, k, ctx->stream);
       eng.item_sq = nullptr;
       eng.sq_step = 0;
@@ -740,6 +766,25 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
     }
   }
   return eng.phase(batch, tau, R, U);
+}
+
+// C = opA(A) B in FP64 (report and re-orthonormalisation products): from digits where the
+// engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`.
+int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const double* B, double* C) {
+  const long long md = mat_doubles(eng.d);
+  AddTerms none;
+  Engine e{ctx, eng.d, MG_PREC_FP64, 0};
+  if (!e.digits64()) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
+  void *ab, *bb, *sums;
+  MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, batch), &ab));
+  MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(e.d, batch), &bb));
+  MG_TRY(ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms), &sums));
+  if (eng.abuf) eng.abuf = ab;   // the slots may have grown
+  if (eng.bbuf[0]) eng.bbuf[0] = bb;
+  const SplitCtl c = e.ctl();
+  MG_TRY(f64d_slice_a(e.d, batch, A, md, opA, ab, ctx->stream, c));
+  MG_TRY(f64d_slice_b(e.d, batch, B, md, bb, ctx->stream, c));
+  return f64d_gemm(e.d, batch, opA, A, md, ab, B, md, bb, C, md, none, sums, ctx->sms, ctx->status, ctx->stream, c);
 }
 
 // One Newton-Schulz polar step in FP64 on a batch: Z <- Z (3I - Z^dag Z)/2.
@@ -753,12 +798,11 @@ int reorth_batch(mg_ctx* ctx, Engine& eng, int batch, double* Z, long long sZ) {
   MG_TRY(ws(ctx, WS_NS_G, md * batch, &G));
   MG_TRY(ws(ctx, WS_NS_H, md * batch, &H));
   MG_TRY(eng.to_fp64(batch, Z, sZ, Zf, md));
-  AddTerms none;
-  MG_TRY(launch_cgemm_f64(batch, d, Zf, md, 1, Zf, md, G, md, none, ctx->stream));
+  MG_TRY(mul_f64(ctx, eng, batch, 1, Zf, Zf, G));
   const double* src[1] = {G};
   double cf[1] = {-0.5};
   MG_TRY(launch_lincomb(batch, d, H, 1, src, cf, 1.5, ctx->stream));
-  MG_TRY(launch_cgemm_f64(batch, d, Zf, md, 0, H, md, G, md, none, ctx->stream));
+  MG_TRY(mul_f64(ctx, eng, batch, 0, Zf, H, G));
   return eng.from_fp64(batch, G, md, Z, sZ);
 }
 
@@ -808,6 +852,7 @@ size_t per_interval_bytes(int d, int prec, int L) {
   size_t md = (size_t)mat_doubles(d) * sizeof(double);
   size_t b = 10 * md;   // (one more for the gathered pairs of a segmented tree)
   if (prec == MG_PREC_SPLIT) b += split_a_bytes(d, L, 1) + 2 * split_b_bytes(d, L, 1);
+  else if (d >= kF64DigitsMinDim) b += f64d_a_bytes(d, 1) + 2 * f64d_b_bytes(d, 1);
   return b;
 }
 
@@ -1164,6 +1209,7 @@ int mg_ctx_create(mg_ctx** out, int device, void* stream) {
   mg_ctx* c = new mg_ctx();
   c->device = device;
   c->stream = reinterpret_cast<cudaStream_t>(stream);
+  c->sms = prop.multiProcessorCount;
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -1532,6 +1578,9 @@ int mg_cgemm(mg_ctx* ctx, int batch, int d, const double* A, const double* B, do
   MG_TRY(validate_prec(precision, slices));
   MG_CUDA_TRY(cudaSetDevice(ctx->device));
   Engine eng{ctx, d, precision, slices};
+  // arbitrary operands: FP64's error bound is relative to |A| |B| entry by entry, the
+  // digits' to the largest entries of A's row and B's column
+  eng.fp64_pipe = true;
   const long long md = mat_doubles(d);
   const int chunk = std::min(chunk_size(ctx, d, precision, slices, batch, 1), 65535);
   for (int b0 = 0; b0 < batch; b0 += chunk) {
@@ -1714,8 +1763,7 @@ int finish_prop(mg_ctx* ctx, Engine& eng, PropState& ps, double* out, int flags,
     } else {
       double* G;
       MG_TRY(ws(ctx, WS_NS_G, md, &G));
-      AddTerms none;
-      MG_TRY(launch_cgemm_f64(1, d, accf, md, 1, accf, md, G, md, none, ctx->stream));
+      MG_TRY(mul_f64(ctx, eng, 1, 1, accf, accf, G));
       MG_TRY(launch_max_identity_defect(1, d, G, sc, ctx->stream));
     }
     MG_CUDA_TRY(cudaMemcpyAsync(&rep->unitarity_defect, sc, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1816,7 +1864,8 @@ int mg_evolve(mg_plan* p, int output, const double* in, double* out, int reorth_
     rep->max_norm1 = st.max_norm;
     rep->matrix_products = eng.products;
   }
-  if (p->precision == MG_PREC_SPLIT) return check_status(ctx);
+  if (p->precision == MG_PREC_SPLIT || (eng.digits64() && (rep || (flags & MG_FLAG_HOST_PTRS))))
+    return check_status(ctx);
   if (flags & MG_FLAG_HOST_PTRS) MG_CUDA_TRY(cudaStreamSynchronize(s));
   return MG_OK;
 }
@@ -3153,7 +3202,7 @@ void server_loop(mg_server* srv) {
     }
     ExpmStats st;
     if (fill > 0) rc = process_chunk(ctx, eng, segs, fill, 0, srv->segs_dev, srv->psi_dev, &st);
-    if (rc == MG_OK && eng.prec == MG_PREC_SPLIT) rc = check_status(ctx);
+    if (rc == MG_OK && (eng.prec == MG_PREC_SPLIT || eng.digits64())) rc = check_status(ctx);
     // completed jobs leave; on an error every job of the group fails
     std::vector<SJob*> done_now;
     for (SJob* j : group)

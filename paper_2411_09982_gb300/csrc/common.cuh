@@ -126,6 +126,9 @@ struct AddTerms {
   // FP64 product only: with item_sq set, items with item_sq[b] <= sq_step are skipped
   const int* item_sq = nullptr;
   int sq_step = 0;
+  // FP64 product only: with only_a and only_b set, items with both marks zero are skipped
+  const int* only_a = nullptr;
+  const int* only_b = nullptr;
 };
 int launch_cgemm_f64(int batch, int d, const double* A, long long strideA, int opA,
                      const double* B, long long strideB, double* C, long long strideC,
@@ -179,6 +182,21 @@ int split_slice_sym(int d, int L, int batch, const double* M, long long sM, void
 int split_sym_fill(int d, int batch, double* C, long long sC, cudaStream_t s);
 int split_gemm(int d, int L, int batch, const void* abuf, const void* bbuf, double* C, long long sC,
                const AddTerms& add, int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
+
+// FP64 products from integer digits on the tensor cores; see gemm_f64_digits.cu.  Operand
+// buffers are filled by the slicers (opA: 0 = A, 1 = A^dagger); the product also takes the
+// operands themselves, for items the slicers marked as outside the digits' range, so C
+// must not alias them.  scratch: f64d_scratch_bytes(sms) of device memory.
+size_t f64d_a_bytes(int d, int batch);
+size_t f64d_b_bytes(int d, int batch);
+size_t f64d_scratch_bytes(int sms);
+int f64d_slice_a(int d, int batch, const double* A, long long sA, int opA, void* buf, cudaStream_t s,
+                 const SplitCtl& ctl = SplitCtl());
+int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cudaStream_t s,
+                 const SplitCtl& ctl = SplitCtl());
+int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const void* abuf, const double* B,
+              long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
+              int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
 
 // State propagation; see propagate.cu.
 int launch_state_chain(int n_steps, int d, const double* U, long long sU, double* psi, double* tmp,

@@ -23,6 +23,8 @@ struct AddDev {
   double scale;
   const int* item_sq;   // null, or per-item squaring counts: item b is skipped when item_sq[b] <= sq_step
   int sq_step;
+  const int* only_a;    // null, or per-item marks: item b is skipped when only_a[b] and only_b[b] are zero
+  const int* only_b;
 };
 
 template <int TM>
@@ -37,6 +39,7 @@ cgemm_f64_kernel(int d, const double* __restrict__ A, long long sA, int opA,
 
   const int b = blockIdx.z;
   if (add.item_sq && add.item_sq[b] <= add.sq_step) return;   // uniform over the CTA
+  if (add.only_a && (add.only_a[b] | add.only_b[b]) == 0) return;
   const double2* Ab = reinterpret_cast<const double2*>(A + b * sA);
   const double2* Bb = reinterpret_cast<const double2*>(B + b * sB);
   const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TM;
@@ -135,6 +138,8 @@ int launch_cgemm_f64(int batch, int d, const double* A, long long strideA, int o
   a.scale = add.scale;
   a.item_sq = add.item_sq;
   a.sq_step = add.sq_step;
+  a.only_a = add.only_a;
+  a.only_b = add.only_b;
   // tile edge: the smallest of 16, 32, 64 that covers d (64 beyond)
   if (d <= 16) {
     cgemm_f64_kernel<16><<<dim3(1, 1, batch), 256, 0, s>>>(d, A, strideA, opA, B, strideB, C, strideC, a);

@@ -47,6 +47,7 @@
 // memory while a tensor-core operation or a copy into it is still in flight.
 #include "common.cuh"
 #include "df32.cuh"
+#include "tc_ptx.cuh"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -501,182 +502,6 @@ slice_b_kernel(int d, int Kp, int Np, int beta, const double* __restrict__ B, lo
   // rows d..Np/2 of every plane are never read: the tensor map ends at row d (TMA fills zeros)
 }
 
-// ---------------------------------------------------------------------------
-// PTX wrappers
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Poll until the phase of `parity` completes or the deadline passes.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t deadline) {
-  while (!mbar_try_wait(bar, parity)) {
-    if (global_ns() > deadline) return false;
-  }
-  return true;
-}
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
-                                            int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
-                                            int c2, int c3, int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(bar))
-      : "memory");
-}
-// CTA-pair forms (cta_group::2): the copy may signal the barrier of either CTA of the pair
-__device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster, int c0,
-                                                 int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar_cluster)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_5d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster, int c0,
-                                                 int c1, int c2, int c3, int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar_cluster)
-      : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// shared::cluster address of this CTA's variable `p` as it lies in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                 uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// arrive on the barrier at this offset in both CTAs of the pair once the issued MMAs
-// complete: one commit per CTA, each naming that CTA's barrier by its cluster address
-__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   cluster_addr(bar, 0))
-               : "memory");
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   cluster_addr(bar, 1))
-               : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptor: K-major operand tile, 64-byte swizzle,
-// 8-row core groups 512 bytes apart (rows are 64 bytes), descriptor version 1.
-// The second K = 16 step of a 64-byte row starts 32 bytes further: the swizzle
-// is applied to the final address bits, so advancing the start address inside
-// the atom selects the next 16 elements of every row.
-__device__ __forceinline__ uint64_t sw64_kmajor_desc(uint32_t saddr) {
-  uint64_t desc = 0;
-  desc |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  desc |= (uint64_t)1 << 16;            // leading-dimension offset (unused with swizzle)
-  desc |= (uint64_t)(512 >> 4) << 32;   // stride-dimension offset
-  desc |= (uint64_t)1 << 46;            // descriptor version
-  desc |= (uint64_t)4 << 61;            // SWIZZLE_64B
-  return desc;
-}
-
-// The same for 32-byte rows: SWIZZLE_32B, 8-row core groups 256 bytes apart.
-__device__ __forceinline__ uint64_t sw32_kmajor_desc(uint32_t saddr) {
-  uint64_t desc = 0;
-  desc |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  desc |= (uint64_t)1 << 16;            // leading-dimension offset (unused with swizzle)
-  desc |= (uint64_t)(256 >> 4) << 32;   // stride-dimension offset
-  desc |= (uint64_t)1 << 46;            // descriptor version
-  desc |= (uint64_t)6 << 61;            // SWIZZLE_32B
-  return desc;
-}
-// The same for 128-byte rows: SWIZZLE_128B, 8-row core groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t sw128_kmajor_desc(uint32_t saddr) {
-  uint64_t desc = 0;
-  desc |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  desc |= (uint64_t)1 << 16;            // leading-dimension offset (unused with swizzle)
-  desc |= (uint64_t)(1024 >> 4) << 32;  // stride-dimension offset
-  desc |= (uint64_t)1 << 46;            // descriptor version
-  desc |= (uint64_t)2 << 61;            // SWIZZLE_128B
-  return desc;
-}
 template <int BK>
 __device__ __forceinline__ uint64_t kmajor_desc(uint32_t saddr) {
   return BK == 64 ? sw128_kmajor_desc(saddr) : (BK == 32 ? sw64_kmajor_desc(saddr) : sw32_kmajor_desc(saddr));
@@ -1178,7 +1003,7 @@ static int get_encoder() {
 // 4-D map over digit tiles: (k, row, slice, batch), box (32, box_rows, box_slices, 1), SWIZZLE_64B.
 // B digits: dims {Kh, d valid rows (of Np / 2 allocated), 3 planes, L, batch};
 // box {32, 64, planes, digits, 1}; rows from d on read as zeros
-static int make_bplane_map(CUtensorMap* map, const void* base, int Kh, int rows, int valid_rows, int L, int batch,
+int make_bplane_map(CUtensorMap* map, const void* base, int Kh, int rows, int valid_rows, int L, int batch,
                            int box_planes, int box_digits, int bk) {
   MG_TRY(get_encoder());
   cuuint64_t dims[5] = {(cuuint64_t)Kh, (cuuint64_t)valid_rows, 3, (cuuint64_t)L, (cuuint64_t)batch};
@@ -1198,8 +1023,8 @@ static int make_bplane_map(CUtensorMap* map, const void* base, int Kh, int rows,
   return MG_OK;
 }
 // A digits: dims {Kp, d valid rows (of `rows` allocated), L, batch}; rows from d on read as zeros
-static int make_digit_map(CUtensorMap* map, const void* base, int Kp, int rows, int valid_rows, int L, int batch,
-                          int bk, int box_rows = SG_BM, int box_slices = -1) {
+int make_digit_map(CUtensorMap* map, const void* base, int Kp, int rows, int valid_rows, int L, int batch,
+                          int bk, int box_rows, int box_slices) {
   MG_TRY(get_encoder());
   cuuint64_t dims[4] = {(cuuint64_t)Kp, (cuuint64_t)valid_rows, (cuuint64_t)L, (cuuint64_t)batch};
   cuuint64_t strides[3] = {(cuuint64_t)Kp * 2, (cuuint64_t)rows * Kp * 2, (cuuint64_t)L * rows * Kp * 2};
