@@ -2,12 +2,15 @@
 // product U_{N-1} ... U_0 psi0), with the optional FP64 renormalisation
 // psi <- psi / |psi| every R intervals.
 //
-// Small d (<= 256): one CTA carries the state through all intervals of a
-// chunk: psi lives in shared memory, each warp forms whole rows of U_n psi_n
-// (coalesced row reads of U_n), one barrier per interval.  The chain is
-// latency-bound; its traffic is one read of every U_n.
+// d <= 32: one CTA carries the state through all intervals of a chunk: psi lives in
+// shared memory, each warp forms whole rows of U_n psi_n (coalesced row reads of U_n), one
+// barrier per interval.
+// 32 < d <= 256: a cluster of C CTAs shares the rows of one state; every CTA holds all of
+// psi, and a finished row is written into every CTA's copy (chain_cluster_kernel).
 // Large d: one multi-CTA matrix-vector launch per interval (HBM-bound).
 #include "common.cuh"
+
+#include <mutex>
 
 namespace mg {
 
@@ -86,6 +89,108 @@ multi_chain_kernel(int d, const ChainSeg* __restrict__ segs, const double* __res
   chain_body(g.count, d, U + g.first * sU, sU, psi[g.job], reorth_every, g.done_before, sh, red, nullptr);
 }
 
+// The chain of one job on a cluster: CTA r of C holds rows [r d / C, (r + 1) d / C), one row
+// per warp (more only where the device schedules no cluster of the wanted size), and a copy
+// of psi.  A row is read from U_n into registers one interval ahead (the loads do not depend
+// on psi), multiplied in the same order as in chain_body (lanes strided by 32, then the
+// butterfly), and stored into all C copies through distributed shared memory; one cluster
+// barrier per interval.  Bound by the FP64 pipe of the cluster's SMs (4 d^2 / C FMAs each)
+// and the barrier: the single CTA took 88 us per interval at d = 256, of which 16 SMs leave
+// 5.  C: rows per CTA down to 8-16, where the barrier (~0.7 us) weighs as much as the row.
+__global__ void __launch_bounds__(512)
+chain_cluster_kernel(int d, int n_steps, const ChainSeg* __restrict__ segs, const double* __restrict__ U, long long sU,
+                     double* psi_one, double* const* __restrict__ psi_many, int reorth_every, int step_offset,
+                     double* __restrict__ traj) {
+  __shared__ double2 buf[2][256];
+  __shared__ double red[16];
+  uint32_t rank, C;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(C));
+  double* psi = psi_one;
+  if (segs) {
+    const ChainSeg g = segs[blockIdx.x / C];
+    n_steps = g.count;
+    U += g.first * sU;
+    psi = psi_many[g.job];
+    step_offset = g.done_before;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int r0 = (int)((long long)d * rank / C), r1 = (int)((long long)d * (rank + 1) / C);
+  const int first = r0 + warp;
+  for (int i = threadIdx.x; i < d; i += blockDim.x) buf[0][i] = reinterpret_cast<double2*>(psi)[i];
+  double2 u[8];   // this warp's first row of the interval, d <= 256
+  auto fetch = [&](int n) {
+    const double2* row = reinterpret_cast<const double2*>(U + n * sU) + (long long)first * d;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[q] = (first < r1 && q * 32 + lane < d) ? row[q * 32 + lane] : make_double2(0.0, 0.0);
+  };
+  if (n_steps > 0) fetch(0);
+  // every CTA has read psi before any may write it back, and has started before a remote store
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  int cur = 0;
+  for (int n = 0; n < n_steps; ++n) {
+    for (int i = first; i < r1; i += nw) {
+      double re = 0.0, im = 0.0;
+      if (i == first) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (q * 32 + lane < d) {
+            const double2 v = buf[cur][q * 32 + lane];
+            re = fma(u[q].x, v.x, re);
+            re = fma(-u[q].y, v.y, re);
+            im = fma(u[q].x, v.y, im);
+            im = fma(u[q].y, v.x, im);
+          }
+        }
+        if (n + 1 < n_steps) fetch(n + 1);
+      } else {
+        const double2* row = reinterpret_cast<const double2*>(U + n * sU) + (long long)i * d;
+        for (int j = lane; j < d; j += 32) {
+          const double2 w = row[j], v = buf[cur][j];
+          re = fma(w.x, v.x, re);
+          re = fma(-w.y, v.y, re);
+          im = fma(w.x, v.y, im);
+          im = fma(w.y, v.x, im);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+      }
+      if (lane < (int)C) {   // lane q stores into CTA q's copy
+        const uint32_t a = (uint32_t)__cvta_generic_to_shared(&buf[cur ^ 1][i]);
+        uint32_t ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"((uint32_t)lane));
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(re), "d"(im) : "memory");
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cur ^= 1;
+    const int done = step_offset + n + 1;
+    if (reorth_every > 0 && done % reorth_every == 0) {   // every CTA on its own copy
+      double s = 0.0;
+      for (int i = threadIdx.x; i < d; i += blockDim.x) s += buf[cur][i].x * buf[cur][i].x + buf[cur][i].y * buf[cur][i].y;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) red[warp] = s;
+      __syncthreads();
+      if (warp == 0) {
+        double v = lane < nw ? red[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[0] = v;
+      }
+      __syncthreads();
+      const double inv = 1.0 / sqrt(red[0]);
+      for (int i = threadIdx.x; i < d; i += blockDim.x) { buf[cur][i].x *= inv; buf[cur][i].y *= inv; }
+      __syncthreads();
+    }
+    if (traj) {
+      double2* t_out = reinterpret_cast<double2*>(traj) + (long long)done * d;
+      for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) t_out[i] = buf[cur][i];
+    }
+  }
+  for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) reinterpret_cast<double2*>(psi)[i] = buf[cur][i];
+}
+
 // out = U psi (one interval), rows split over CTAs: 8 warps per CTA, one row per warp.
 __global__ void __launch_bounds__(256)
 matvec_kernel(int d, const double* __restrict__ U, const double* __restrict__ in, double* __restrict__ out) {
@@ -140,12 +245,75 @@ __global__ void norm_defect_kernel(int d, const double* __restrict__ psi, double
   }
 }
 
+static void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int C, int nseg, cudaStream_t s) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)(nseg * C), 1, 1);
+  cfg->blockDim = dim3(512, 1, 1);
+  cfg->stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+// CTAs per state for nseg states of dimension d (32 < d <= 256): about 12 rows per CTA,
+// fewer CTAs where that many clusters do not run at once.  The clusters that fit are asked
+// for once per device and size.
+static int chain_cluster_size(int d, int nseg) {
+  static std::mutex mu;
+  static int fits[64][5];   // clusters of 1 << q CTAs that fit at once, + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  int want = 2;
+  while (want < 16 && want * 12 < d) want *= 2;
+  std::lock_guard<std::mutex> lock(mu);
+  for (int q = 4; q >= 1; --q) {
+    const int C = 1 << q;
+    if (C > want) continue;
+    if (fits[dev][q] == 0) {
+      cudaLaunchConfig_t cfg;
+      cudaLaunchAttribute attr[1];
+      chain_cluster_config(&cfg, attr, C, 1, nullptr);
+      int n = 0;
+      if (ensure_func_attr(reinterpret_cast<const void*>(chain_cluster_kernel),
+                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != MG_OK ||
+          cudaOccupancyMaxActiveClusters(&n, chain_cluster_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+      fits[dev][q] = 1 + n;
+    }
+    if (fits[dev][q] - 1 >= nseg) return C;
+  }
+  return 1;
+}
+
+static int launch_chain_cluster(int C, int nseg, int d, int n_steps, const ChainSeg* segs, const double* U, long long sU,
+                                double* psi, double* const* psi_many, int reorth_every, int step_offset, double* traj,
+                                cudaStream_t s) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  chain_cluster_config(&cfg, attr, C, nseg, s);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, chain_cluster_kernel, d, n_steps, segs, U, sU, psi, psi_many,
+                                           reorth_every, step_offset, traj);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e, "cudaLaunchKernelEx(chain_cluster_kernel)", __FILE__, __LINE__);
+    return MG_ECUDA;
+  }
+  return check_launch("chain_cluster_kernel");
+}
+
 // psi (device, d complex) is carried through n_steps propagators U (stride sU doubles).
 // tmp: d complex of scratch for the large-d path.  traj (may be null): the state
 // after step n is also written to traj + (step_offset + n + 1) d complex.
 int launch_state_chain(int n_steps, int d, const double* U, long long sU, double* psi, double* tmp,
                        int reorth_every, int step_offset, cudaStream_t s, double* traj) {
   if (n_steps <= 0) return MG_OK;
+  const int C = d > 32 && d <= 256 && n_steps > 1 ? chain_cluster_size(d, 1) : 1;
+  if (C > 1)
+    return launch_chain_cluster(C, 1, d, n_steps, nullptr, U, sU, psi, nullptr, reorth_every, step_offset, traj, s);
   if (d <= 256) {
     int threads = d <= 32 ? ((d + 31) / 32) * 32 * 8 : CHAIN_THREADS;
     if (threads > CHAIN_THREADS) threads = CHAIN_THREADS;
@@ -176,6 +344,11 @@ int launch_multi_chain(int nseg, int d, const ChainSeg* segs_dev, const double* 
                        double* const* psi_dev, int reorth_every, cudaStream_t s) {
   if (nseg <= 0) return MG_OK;
   if (d > 256) return MG_EUNSUPPORTED;
+  // clusters while all states' clusters run at once; beyond, one CTA per state keeps the
+  // device as busy without the barriers
+  const int C = d > 32 ? chain_cluster_size(d, nseg) : 1;
+  if (C > 1)
+    return launch_chain_cluster(C, nseg, d, 0, segs_dev, U, sU, nullptr, psi_dev, reorth_every, 0, nullptr, s);
   const int threads = d <= 32 ? 256 : CHAIN_THREADS;
   multi_chain_kernel<<<nseg, threads, sizeof(double2) * 2 * d, s>>>(d, segs_dev, U, sU, psi_dev, reorth_every);
   return check_launch("multi_chain_kernel");
