@@ -715,9 +715,7 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   AddTerms rest = add;
   rest.item_sq = ctl.item_sq;
   rest.sq_step = ctl.sq_step;
-  rest.only_a = a.bad;
-  rest.only_b = b.bad;
-  return launch_cgemm_f64(batch, d, A, sA, opA, B, sB, C, sC, rest, s);
+  return launch_cgemm_f64_marked(batch, d, A, sA, opA, B, sB, C, sC, rest, a.bad, b.bad, sms, s);
 }
 
 }  // namespace mg
