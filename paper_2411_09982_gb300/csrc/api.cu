@@ -158,6 +158,7 @@ struct mg_plan {
   int* csr_diag = nullptr;       // position of each row's diagonal entry
   double* csr_val = nullptr;     // (1 + K) x nnz complex, operator-major
   long long csr_nnz = 0;
+  bool csr_real = false;
   std::vector<int> csr_rowptr_h;  // host copies of the pattern (cluster partitioning, send masks)
   std::vector<int> csr_col_h;
   // ||H - tau I||_1 of H0 and the Kx operators padded to dimension opnorm_dp (bounds of
@@ -880,6 +881,7 @@ namespace {
 struct CsrHost {
   std::vector<int> rowptr, col, diag;
   std::vector<double> val;   // (1 + K) x nnz complex
+  bool real = true;          // every value's imaginary part is zero
 };
 void build_csr_host(const double* dense, int d, int nops, CsrHost& h) {
   const size_t dd = (size_t)d * d;
@@ -901,6 +903,7 @@ void build_csr_host(const double* dense, int d, int nops, CsrHost& h) {
     h.rowptr[i + 1] = (int)h.col.size();
   }
   const size_t nnz = h.col.size();
+  h.real = true;
   h.val.assign((size_t)nops * nnz * 2, 0.0);
   for (int op = 0; op < nops; ++op)
     for (int i = 0; i < d; ++i)
@@ -908,6 +911,7 @@ void build_csr_host(const double* dense, int d, int nops, CsrHost& h) {
         const double* v = dense + (size_t)op * 2 * dd + 2 * ((size_t)i * d + h.col[e]);
         h.val[2 * ((size_t)op * nnz + e)] = v[0];
         h.val[2 * ((size_t)op * nnz + e) + 1] = v[1];
+        h.real = h.real && v[1] == 0.0;
       }
 }
 int check_action_limits(int d, int nops) {
@@ -949,6 +953,7 @@ int ensure_csr(mg_plan* p) {
   MG_TRY(up(reinterpret_cast<void**>(&p->csr_diag), h.diag.data(), sizeof(int) * h.diag.size()));
   MG_TRY(up(reinterpret_cast<void**>(&p->csr_val), h.val.data(), sizeof(double) * h.val.size()));
   p->csr_nnz = (long long)h.col.size();
+  p->csr_real = h.real;
   p->csr_rowptr_h = h.rowptr;
   p->csr_col_h = h.col;
   p->csr_ok = true;
@@ -966,6 +971,7 @@ ActionJob action_job(mg_plan* p, double* psi) {
   j.col = p->csr_col;
   j.diag = p->csr_diag;
   j.val = p->csr_val;
+  j.real_ops = p->csr_real;
   j.c = p->c;
   j.psi = psi;
   return j;
@@ -981,9 +987,59 @@ struct CsrRef {
 struct ActionShape {
   std::vector<size_t> order;
   int dmax = 1, nmax = 0, cluster = 1, cap = 0;
+  int row_regs = 0;              // real-row kernel: nonzeros of a row held in registers (0: the general kernels)
   size_t rec_doubles = 0, mat_doubles = 0, mask_words = 0;
   std::vector<uint16_t> masks;   // launch order, d per job (cluster variant)
 };
+// Workspace sizes and send masks of a chosen shape.
+void finish_shape(const std::vector<ActionJob>& jobs, const std::vector<CsrRef>& pat, ActionShape& S) {
+  const size_t nj = jobs.size();
+  S.rec_doubles = 0;
+  S.mat_doubles = 0;
+  S.mask_words = 0;
+  for (auto& j : jobs) {
+    S.rec_doubles += (size_t)j.N * ACTION_REC;
+    if (!S.row_regs && (S.cluster > 1 || j.nnz > S.cap)) S.mat_doubles += 2 * (size_t)j.nnz;
+    if (S.cluster > 1) S.mask_words += (size_t)j.d;
+  }
+  // send masks of the cluster variant: row j goes to every CTA with a nonzero in column j
+  S.masks.assign(S.mask_words, 0);
+  if (S.cluster > 1) {
+    size_t off = 0;
+    for (size_t q = 0; q < nj; ++q) {
+      const size_t jq = S.order[q];
+      const std::vector<int>& rp = *pat[jq].rowptr;
+      const std::vector<int>& col = *pat[jq].col;
+      const int d = jobs[jq].d, per = (d + S.cluster - 1) / S.cluster;
+      for (int i = 0; i < d; ++i)
+        for (int e = rp[i]; e < rp[i + 1]; ++e) S.masks[off + col[e]] |= (uint16_t)(1u << (i / per));
+      off += (size_t)d;
+    }
+  }
+}
+// The real-row kernel (action_rows_kernel): every job with real operators and rows of at
+// most 24 nonzeros, at most 256 rows per CTA.
+bool shape_action_rows(const std::vector<ActionJob>& jobs, const std::vector<CsrRef>& pat, ActionShape& S) {
+  const size_t nj = jobs.size();
+  int longest = 0;
+  for (size_t q = 0; q < nj; ++q) {
+    if (!jobs[q].real_ops) return false;
+    const std::vector<int>& rp = *pat[q].rowptr;
+    for (int i = 0; i < jobs[q].d; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
+  }
+  if (longest > 24) return false;
+  // at most 64 rows per CTA where a cluster of 16 reaches that: below, the cluster barrier
+  // outweighs the FP64 work it divides, above, one SM's FP64 pipe bounds the application
+  // (64 uneven jobs of d <= 256: 200 ms with one CTA per job, 157 with 128 rows, 135 with 64,
+  // 143 with 32; one job of d = 256: 165, 118, 96, 96; the general kernels: 259 and 189)
+  int want = 1;
+  while (want < 16 && want * 64 < S.dmax) want *= 2;
+  S.cap = 0;
+  S.cluster = want > 1 ? action_cluster_size(want, S.dmax, 0) : 1;
+  if ((S.dmax + S.cluster - 1) / S.cluster > 256) return false;
+  S.row_regs = longest <= 8 ? 8 : longest <= 16 ? 16 : 24;
+  return true;
+}
 // A few large jobs run as one thread block cluster each (up to 16 CTAs, about
 // 1024 nonzeros per CTA or more, every job's cluster resident at once);
 // otherwise one CTA per job.
@@ -999,6 +1055,11 @@ void shape_action(const std::vector<ActionJob>& jobs, const std::vector<CsrRef>&
     S.dmax = std::max(S.dmax, j.d);
     S.nmax = std::max(S.nmax, j.N);
     nnz_max = std::max(nnz_max, j.nnz);
+  }
+  S.row_regs = 0;
+  if (shape_action_rows(jobs, pat, S)) {
+    finish_shape(jobs, pat, S);
+    return;
   }
   int want = 1;
   while (want < 16 && 2 * want * 512 <= nnz_max && (size_t)(2 * want) * nj <= 152) want *= 2;
@@ -1030,28 +1091,7 @@ void shape_action(const std::vector<ActionJob>& jobs, const std::vector<CsrRef>&
     for (auto& j : jobs)
       if (j.nnz > S.cap && action_smem_bytes(S.dmax, j.nnz) <= budget) S.cap = j.nnz;
   }
-  S.rec_doubles = 0;
-  S.mat_doubles = 0;
-  S.mask_words = 0;
-  for (auto& j : jobs) {
-    S.rec_doubles += (size_t)j.N * ACTION_REC;
-    if (S.cluster > 1 || j.nnz > S.cap) S.mat_doubles += 2 * (size_t)j.nnz;
-    if (S.cluster > 1) S.mask_words += (size_t)j.d;
-  }
-  // send masks of the cluster variant: row j goes to every CTA with a nonzero in column j
-  S.masks.assign(S.mask_words, 0);
-  if (S.cluster > 1) {
-    size_t off = 0;
-    for (size_t q = 0; q < nj; ++q) {
-      const size_t jq = S.order[q];
-      const std::vector<int>& rp = *pat[jq].rowptr;
-      const std::vector<int>& col = *pat[jq].col;
-      const int d = jobs[jq].d, per = (d + S.cluster - 1) / S.cluster;
-      for (int i = 0; i < d; ++i)
-        for (int e = rp[i]; e < rp[i + 1]; ++e) S.masks[off + col[e]] |= (uint16_t)(1u << (i / per));
-      off += (size_t)d;
-    }
-  }
+  finish_shape(jobs, pat, S);
 }
 // Launch-ordered records with their interval-record and matrix pointers set.
 void layout_action(const std::vector<ActionJob>& jobs, const ActionShape& S, double* rec, double* mat,
@@ -1063,7 +1103,7 @@ void layout_action(const std::vector<ActionJob>& jobs, const ActionShape& S, dou
     j.cheb = rec + ro;
     ro += (size_t)j.N * ACTION_REC;
     j.abuf = nullptr;
-    if (S.cluster > 1 || j.nnz > S.cap) {
+    if (!S.row_regs && (S.cluster > 1 || j.nnz > S.cap)) {
       j.abuf = mat + mo;
       mo += 2 * (size_t)j.nnz;
     }
@@ -1108,7 +1148,7 @@ int run_action(mg_ctx* ctx, std::vector<ActionJob>& jobs, const std::vector<CsrR
   MG_CUDA_TRY(cudaMemcpyAsync(dev, launch.data(), sizeof(ActionJob) * nj, cudaMemcpyHostToDevice, ctx->stream));
   int e0 = -1, e1 = -1;
   if (ctx->timing) MG_TRY(timing_mark(ctx, &e0));
-  MG_TRY(launch_action_chain((int)nj, dev, S.dmax, S.nmax, S.cap, S.cluster, ctx->stream));
+  MG_TRY(launch_action_chain((int)nj, dev, S.dmax, S.nmax, S.cap, S.cluster, S.row_regs, ctx->stream));
   if (ctx->timing) {
     MG_TRY(timing_mark(ctx, &e1));
     ctx->ev_pending.emplace_back(e0, e1);
@@ -3041,7 +3081,7 @@ int issue_action_slice(mg_server* srv, SActionGroup& g, bool bounds) {
   ActionJob* dev = reinterpret_cast<ActionJob*>(reinterpret_cast<char*>(g.mem) + g.off_jobs);
   MG_CUDA_TRY(cudaMemcpyAsync(dev, g.xfer.data(), sizeof(ActionJob) * g.xfer.size(), cudaMemcpyHostToDevice, s));
   MG_TRY(launch_action_chain((int)g.xfer.size(), dev, g.shape.dmax, bounds ? g.shape.nmax : 0, g.shape.cap,
-                             g.shape.cluster, s));
+                             g.shape.cluster, g.shape.row_regs, s));
   if (!g.done) MG_CUDA_TRY(cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming));
   MG_CUDA_TRY(cudaEventRecord(g.done, s));
   return MG_OK;
@@ -3420,6 +3460,7 @@ int submit_action(mg_server* srv, const mg_job* job, uint64_t* job_id) {
     a.col = reinterpret_cast<const int*>(col);
     a.diag = reinterpret_cast<const int*>(dg);
     a.val = reinterpret_cast<const double*>(val);
+    a.real_ops = h.real;
     a.c = reinterpret_cast<const double*>(c);
     a.psi = reinterpret_cast<double*>(psi);
     return r;

@@ -237,6 +237,7 @@ struct ActionJob {
   double* psi;          // d complex, in and out
   double* traj;         // null, or (first + N + 1) x d complex: the state after interval n at row first + n + 1
   const uint16_t* sendmask;  // cluster variant: per row, bit q set if CTA q reads that row
+  int real_ops;         // every operator value is real (host-side choice of the kernel)
   int status;           // MG_OK, or set by the kernel when the job stopped early
   long long max_steps;  // operator applications after which a launch stops at an interval end (0: none)
   int done;             // written by the kernel: intervals this launch completed
@@ -255,7 +256,9 @@ int action_cluster_size(int want, int dmax, int cap_loc);
 // bounds kernel, then the chain: one CTA per job (cluster <= 1, nnz_cap = the
 // nonzeros held on chip) or one cluster of `cluster` CTAs per job (nnz_cap =
 // own-row nonzeros held on chip per CTA)
-int launch_action_chain(int njobs, ActionJob* jobs_dev, int dmax, int nmax, int nnz_cap, int cluster,
+// row_regs != 0 (8, 16 or 24, at least the longest row of any job; every job with real
+// operators, at most 256 rows per CTA): the real-row kernel on clusters of any size
+int launch_action_chain(int njobs, ActionJob* jobs_dev, int dmax, int nmax, int nnz_cap, int cluster, int row_regs,
                         cudaStream_t s);
 
 // dst (dp x dp, zero padded) <- src (d x d), for `count` stacked matrices
