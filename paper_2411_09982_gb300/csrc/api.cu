@@ -525,6 +525,32 @@ struct Engine {
     return MG_OK;
   }
   int timing_begin(int* idx) { return timing_mark(ctx, idx); }
+  // real products on the lower triangle that degree m and sq squarings take
+  static int real_products(int m, int sq) {
+    const int kc = m / 2, ks = (m - 1) / 2, p = (kc + 1) / 2;
+    return p + (kc > p) + (ks > p) + 1 + 2 * sq;
+  }
+  // FP64 exponentials in one launch (expm_small.cu)
+  bool small64() const { return prec == MG_PREC_FP64 && d <= expm_small_max_dim(); }
+  // per_poly products of the polynomial and sq squarings (sq_dev: per item, at most sq) are
+  // counted as complex products, as the step-by-step form issues them
+  int expm_small(int batch, const double* W, const double* tau, int m, int p, int per_poly, int sq, const int* sq_dev,
+                 double* U) {
+    products += (long long)batch * (per_poly + sq);
+    int e0 = -1, e1 = -1;
+    if (ctx->timing) MG_TRY(timing_begin(&e0));
+    MG_TRY(launch_expm_small(batch, d, W, tau, m, p, sq, sq_dev, x_sym ? 1 : 0, U, ctx->stream));
+    if (ctx->timing) {
+      MG_TRY(timing_begin(&e1));
+      ctx->ev_pending.emplace_back(e0, e1);
+      ctx->t_launches += 1;
+      // the flops issued: real products of the lower triangle, or complex ones
+      const double work = x_sym ? (double)d * d * (d + 1) * real_products(m, sq_dev ? 0 : sq)
+                                : 8.0 * d * d * d * (per_poly + (sq_dev ? 0 : sq));
+      ctx->t_flops += work * batch;
+    }
+    return MG_OK;
+  }
   // operand structure of the next split product, where X is known to be imaginary
   void set_structure(int az, int bz) {
     if (x_imag && prec == MG_PREC_SPLIT && (ctx->structure & 1)) {
@@ -709,6 +735,10 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
     }
   }
 
+  if (eng.small64()) {
+    if (sU != md) return MG_EINVAL;
+    return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, tc.s, nullptr, U);
+  }
   // X = -i 2^{-s} W   (in place, into the engine's storage format)
   MG_TRY(eng.scale_x(batch, W, W, tc.s, nullptr, w_df));
   double *R, *Rn;
@@ -738,6 +768,7 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
 int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau, const int* sq_dev,
                    const TaylorChoice& tc, int S, double* U, bool w_df) {
   PhaseRange range("expm");
+  if (eng.small64()) return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, S, sq_dev, U);
   const long long md = mat_doubles(eng.d);
   MG_TRY(eng.scale_x(batch, W, W, 0, sq_dev, w_df));
   double *R, *Rn;
@@ -812,7 +843,10 @@ int reorth_batch(mg_ctx* ctx, Engine& eng, int batch, double* Z, long long sZ) {
 // neighbouring pairs, later item on the left; an odd item is carried up.  Nodes
 // spanning `reorth_span` intervals (a power of two; 0 = never) are
 // re-orthonormalised in FP64.
-int tree_product(mg_ctx* ctx, Engine& eng, int n, const double* U, double** out, int reorth_span) {
+// With `left` set the levels stop at `stop` products or fewer, earliest first from *out on;
+// *left receives their number.
+int tree_product(mg_ctx* ctx, Engine& eng, int n, const double* U, double** out, int reorth_span, int stop = 1,
+                 int* left = nullptr) {
   const int d = eng.d;
   const long long md = mat_doubles(d);
   double *b0, *b1;
@@ -825,7 +859,7 @@ int tree_product(mg_ctx* ctx, Engine& eng, int n, const double* U, double** out,
   }
   const double* cur = U;
   int cnt = n, span = 1, level = 0;
-  while (cnt > 1) {
+  while (cnt > stop) {
     double* dst = (level % 2 == 0) ? b0 : b1;   // level 0 -> ceil(n/2) items, level 1 -> ceil(n/4), ...
     const int pairs = cnt / 2;
     MG_TRY(eng.reserve(pairs));
@@ -843,6 +877,7 @@ int tree_product(mg_ctx* ctx, Engine& eng, int n, const double* U, double** out,
     ++level;
   }
   *out = const_cast<double*>(cur);
+  if (left) *left = cnt;
   return MG_OK;
 }
 
@@ -1701,11 +1736,14 @@ int fold_chunk(mg_ctx* ctx, Engine& eng, PropState& ps, int n, const double* U, 
     MG_TRY(ws(ctx, WS_VEC, 2 * d + 2, &tmp));
     if (!eng.df() && !ps.traj && reorth == 0 && d <= 64 && n >= 8) {
       // small d in FP64: the n dependent matrix-vector steps of the chain are
-      // latency-bound; the chunk's product by the batched tree (log2 n launches
-      // of d^3 products) and one application to psi take less time
-      double* chunk_prod = nullptr;
-      MG_TRY(tree_product(ctx, eng, n, U, &chunk_prod, 0));
-      MG_TRY(launch_state_chain(1, d, chunk_prod, md, ps.psi, tmp + 2, 0, ps.done, ctx->stream));
+      // latency-bound (1.7 us each at d = 30, 0.3 us at d = 2); while a level of the
+      // batched tree, which costs 32 us at d = 30 and 4 us at d = 2 however few products
+      // are left, halves more than 32 steps, it takes less time
+      const int stop = 32;
+      double* prods = const_cast<double*>(U);
+      int left = n;
+      if (n > stop) MG_TRY(tree_product(ctx, eng, n, U, &prods, 0, stop, &left));
+      MG_TRY(launch_state_chain(left, d, prods, md, ps.psi, tmp + 2, 0, ps.done, ctx->stream));
       ps.done += n;
       return MG_OK;
     }

@@ -200,6 +200,14 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
               long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
               int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
 
+// FP64 exponentials of small matrices (d <= expm_small_max_dim()), U_b = e^{-i tau_b}
+// exp(-i W_b) (tau may be null), in one launch; see expm_small.cu.  Degree m and block p as
+// Paterson-Stockmeyer takes them; sq_dev: per-item squaring counts, else sq; real_sym: every
+// W_b is real and symmetric.  W is not modified; U may alias it.
+int expm_small_max_dim();
+int launch_expm_small(int batch, int d, const double* W, const double* tau, int m, int p, int sq, const int* sq_dev,
+                      int real_sym, double* U, cudaStream_t s);
+
 // State propagation; see propagate.cu.
 int launch_state_chain(int n_steps, int d, const double* U, long long sU, double* psi, double* tmp,
                        int reorth_every, int step_offset, cudaStream_t s, double* traj = nullptr);

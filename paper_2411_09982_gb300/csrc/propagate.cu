@@ -2,11 +2,10 @@
 // product U_{N-1} ... U_0 psi0), with the optional FP64 renormalisation
 // psi <- psi / |psi| every R intervals.
 //
-// d <= 32: one CTA carries the state through all intervals of a chunk: psi lives in
-// shared memory, each warp forms whole rows of U_n psi_n (coalesced row reads of U_n), one
-// barrier per interval.
-// 32 < d <= 256: a cluster of C CTAs shares the rows of one state; every CTA holds all of
-// psi, and a finished row is written into every CTA's copy (chain_cluster_kernel).
+// d <= 256: a cluster of C CTAs (one CTA for d <= 32) carries the state through all
+// intervals of a chunk and shares its rows; every CTA holds all of psi in shared memory, and
+// a finished row is written into every CTA's copy (chain_cluster_kernel).  Where more states
+// run at once than their clusters fit, one CTA per state, a warp per row.
 // Large d: one multi-CTA matrix-vector launch per interval (HBM-bound).
 #include "common.cuh"
 
@@ -89,19 +88,23 @@ multi_chain_kernel(int d, const ChainSeg* __restrict__ segs, const double* __res
   chain_body(g.count, d, U + g.first * sU, sU, psi[g.job], reorth_every, g.done_before, sh, red, nullptr);
 }
 
-// The chain of one job on a cluster: CTA r of C holds rows [r d / C, (r + 1) d / C), one row
-// per warp (more only where the device schedules no cluster of the wanted size), and a copy
-// of psi.  A row is read from U_n into registers one interval ahead (the loads do not depend
-// on psi), multiplied in the same order as in chain_body (lanes strided by 32, then the
-// butterfly), and stored into all C copies through distributed shared memory; one cluster
-// barrier per interval.  Bound by the FP64 pipe of the cluster's SMs (4 d^2 / C FMAs each)
-// and the barrier: the single CTA took 88 us per interval at d = 256, of which 16 SMs leave
-// 5.  C: rows per CTA down to 8-16, where the barrier (~0.7 us) weighs as much as the row.
-__global__ void __launch_bounds__(512)
+// The chain of one job on a cluster (C = 1: one CTA): CTA r of C holds rows [r d / C,
+// (r + 1) d / C), T lanes per row, and a copy of psi.  A row is read from U_n into registers
+// AHEAD intervals early (the loads do not depend on psi), multiplied, summed over its T lanes
+// and stored into all C copies through distributed shared memory; one barrier per interval.
+// Bound by the FP64 pipe of the SMs, where a warp's instruction takes about 64 cycles of its
+// quarter: 4 d / T FMAs and 2 log2 T additions per lane.  On one CTA (d <= 32) a warp per row
+// spent as much on the sums as on the products, 6.2 us per interval at d = 30; T = 4 takes
+// 1.7.  On clusters T = 32 is as fast as T = 8 (its loads coalesce better).  At d <= 8 the
+// loads' latency is what an interval takes (0.85 us at d = 2 with one interval ahead), hence
+// AHEAD.  C: rows per CTA down to 8-16, where the barrier (~0.7 us) weighs as much as the rows
+// (one CTA took 88 us per interval at d = 256, of which 16 leave 5).
+template <int T, int Q, int AHEAD>
+__global__ void __launch_bounds__(T == 32 ? 512 : 128)
 chain_cluster_kernel(int d, int n_steps, const ChainSeg* __restrict__ segs, const double* __restrict__ U, long long sU,
                      double* psi_one, double* const* __restrict__ psi_many, int reorth_every, int step_offset,
                      double* __restrict__ traj) {
-  __shared__ double2 buf[2][256];
+  __shared__ double2 buf[2][T * Q];
   __shared__ double red[16];
   uint32_t rank, C;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -115,37 +118,52 @@ chain_cluster_kernel(int d, int n_steps, const ChainSeg* __restrict__ segs, cons
     step_offset = g.done_before;
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int sub = threadIdx.x % T, nrow = blockDim.x / T;
   const int r0 = (int)((long long)d * rank / C), r1 = (int)((long long)d * (rank + 1) / C);
-  const int first = r0 + warp;
+  const int first = r0 + threadIdx.x / T;
+  auto sync = [&]() {
+    if (C > 1)
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else
+      __syncthreads();
+  };
   for (int i = threadIdx.x; i < d; i += blockDim.x) buf[0][i] = reinterpret_cast<double2*>(psi)[i];
-  double2 u[8];   // this warp's first row of the interval, d <= 256
-  auto fetch = [&](int n) {
+  double2 ring[AHEAD][Q];   // this lane's part of its first row: columns sub, sub + T, ...
+  auto fetch = [&](int n, double2 (&u)[Q]) {
+    if (n >= n_steps) return;
     const double2* row = reinterpret_cast<const double2*>(U + n * sU) + (long long)first * d;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) u[q] = (first < r1 && q * 32 + lane < d) ? row[q * 32 + lane] : make_double2(0.0, 0.0);
+    for (int q = 0; q < Q; ++q) u[q] = (first < r1 && q * T + sub < d) ? row[q * T + sub] : make_double2(0.0, 0.0);
   };
-  if (n_steps > 0) fetch(0);
-  // every CTA has read psi before any may write it back, and has started before a remote store
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  int cur = 0;
-  for (int n = 0; n < n_steps; ++n) {
-    for (int i = first; i < r1; i += nw) {
-      double re = 0.0, im = 0.0;
-      if (i == first) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (q * 32 + lane < d) {
-            const double2 v = buf[cur][q * 32 + lane];
+  for (int a = 0; a < AHEAD; ++a) fetch(a, ring[a]);
+  // every CTA has read psi before any may write it back, and has started before a remote store
+  sync();
+  int cur = 0;
+  for (int nb = 0; nb < n_steps; nb += AHEAD)
+#pragma unroll
+  for (int a = 0; a < AHEAD; ++a) {
+    const int n = nb + a;
+    if (n >= n_steps) break;   // uniform over the cluster
+    double2 (&u)[Q] = ring[a];
+    for (int i0 = r0; i0 < r1; i0 += nrow) {   // one round, more only where few CTAs were to be had
+      const int i = i0 + threadIdx.x / T;
+      double re = 0.0, im = 0.0;
+      if (i0 == r0) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          if (q * T < d) {   // uniform; lanes beyond d hold zeros (and read a slot of psi below T Q)
+            const double2 v = q * T + sub < d ? buf[cur][q * T + sub] : make_double2(0.0, 0.0);
             re = fma(u[q].x, v.x, re);
             re = fma(-u[q].y, v.y, re);
             im = fma(u[q].x, v.y, im);
             im = fma(u[q].y, v.x, im);
           }
         }
-        if (n + 1 < n_steps) fetch(n + 1);
-      } else {
+        fetch(n + AHEAD, u);
+      } else if (i < r1) {
         const double2* row = reinterpret_cast<const double2*>(U + n * sU) + (long long)i * d;
-        for (int j = lane; j < d; j += 32) {
+        for (int j = sub; j < d; j += T) {
           const double2 w = row[j], v = buf[cur][j];
           re = fma(w.x, v.x, re);
           re = fma(-w.y, v.y, re);
@@ -153,18 +171,25 @@ chain_cluster_kernel(int d, int n_steps, const ChainSeg* __restrict__ segs, cons
           im = fma(w.y, v.x, im);
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int o = T / 2; o > 0; o >>= 1) {
         re += __shfl_xor_sync(0xffffffffu, re, o);
         im += __shfl_xor_sync(0xffffffffu, im, o);
       }
-      if (lane < (int)C) {   // lane q stores into CTA q's copy
-        const uint32_t a = (uint32_t)__cvta_generic_to_shared(&buf[cur ^ 1][i]);
-        uint32_t ra;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"((uint32_t)lane));
-        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(re), "d"(im) : "memory");
+      if (i < r1) {
+        if (C == 1) {
+          if (sub == 0) buf[cur ^ 1][i] = make_double2(re, im);
+        } else {
+          for (int q = sub; q < (int)C; q += T) {   // the row's lanes share the copies
+            const uint32_t a = (uint32_t)__cvta_generic_to_shared(&buf[cur ^ 1][i]);
+            uint32_t ra;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"((uint32_t)q));
+            asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(re), "d"(im) : "memory");
+          }
+        }
       }
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    sync();
     cur ^= 1;
     const int done = step_offset + n + 1;
     if (reorth_every > 0 && done % reorth_every == 0) {   // every CTA on its own copy
@@ -173,13 +198,9 @@ chain_cluster_kernel(int d, int n_steps, const ChainSeg* __restrict__ segs, cons
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == 0) red[warp] = s;
       __syncthreads();
-      if (warp == 0) {
-        double v = lane < nw ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[0] = v;
-      }
-      __syncthreads();
-      const double inv = 1.0 / sqrt(red[0]);
+      double v = 0.0;
+      for (int w = 0; w < nw; ++w) v += red[w];
+      const double inv = 1.0 / sqrt(v);
       for (int i = threadIdx.x; i < d; i += blockDim.x) { buf[cur][i].x *= inv; buf[cur][i].y *= inv; }
       __syncthreads();
     }
@@ -245,10 +266,21 @@ __global__ void norm_defect_kernel(int d, const double* __restrict__ psi, double
   }
 }
 
-static void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int C, int nseg, cudaStream_t s) {
+using ChainKernel = void (*)(int, int, const ChainSeg*, const double*, long long, double*, double* const*, int, int,
+                             double*);
+// lanes per row, columns per lane and intervals ahead by d
+static ChainKernel chain_kernel(int d) {
+  return d <= 4 ? chain_cluster_kernel<4, 1, 8>
+                : d <= 8 ? chain_cluster_kernel<4, 2, 4>
+                         : d <= 32 ? chain_cluster_kernel<4, 8, 1> : chain_cluster_kernel<32, 8, 1>;
+}
+
+static void chain_cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int d, int C, int nseg,
+                                 cudaStream_t s) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3((unsigned)(nseg * C), 1, 1);
-  cfg->blockDim = dim3(512, 1, 1);
+  const int lanes = (d <= 32 ? 4 : 32) * ceil_div(d, C);
+  cfg->blockDim = dim3(lanes >= 512 ? 512 : (lanes + 31) / 32 * 32, 1, 1);
   cfg->stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
@@ -275,11 +307,12 @@ static int chain_cluster_size(int d, int nseg) {
     if (fits[dev][q] == 0) {
       cudaLaunchConfig_t cfg;
       cudaLaunchAttribute attr[1];
-      chain_cluster_config(&cfg, attr, C, 1, nullptr);
+      // asked of the form with most registers and threads, d = 256
+      const void* k = reinterpret_cast<const void*>(chain_kernel(256));
+      chain_cluster_config(&cfg, attr, 256, C, 1, nullptr);
       int n = 0;
-      if (ensure_func_attr(reinterpret_cast<const void*>(chain_cluster_kernel),
-                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != MG_OK ||
-          cudaOccupancyMaxActiveClusters(&n, chain_cluster_kernel, &cfg) != cudaSuccess) {
+      if (ensure_func_attr(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != MG_OK ||
+          cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
       }
@@ -295,8 +328,10 @@ static int launch_chain_cluster(int C, int nseg, int d, int n_steps, const Chain
                                 cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  chain_cluster_config(&cfg, attr, C, nseg, s);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, chain_cluster_kernel, d, n_steps, segs, U, sU, psi, psi_many,
+  chain_cluster_config(&cfg, attr, d, C, nseg, s);
+  const ChainKernel k = chain_kernel(d);
+  MG_TRY(ensure_func_attr(reinterpret_cast<const void*>(k), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, d, n_steps, segs, U, sU, psi, psi_many,
                                            reorth_every, step_offset, traj);
   if (e != cudaSuccess) {
     set_last_cuda_error(e, "cudaLaunchKernelEx(chain_cluster_kernel)", __FILE__, __LINE__);
@@ -312,13 +347,11 @@ int launch_state_chain(int n_steps, int d, const double* U, long long sU, double
                        int reorth_every, int step_offset, cudaStream_t s, double* traj) {
   if (n_steps <= 0) return MG_OK;
   const int C = d > 32 && d <= 256 && n_steps > 1 ? chain_cluster_size(d, 1) : 1;
-  if (C > 1)
+  if (C > 1 || d <= 32)
     return launch_chain_cluster(C, 1, d, n_steps, nullptr, U, sU, psi, nullptr, reorth_every, step_offset, traj, s);
-  if (d <= 256) {
-    int threads = d <= 32 ? ((d + 31) / 32) * 32 * 8 : CHAIN_THREADS;
-    if (threads > CHAIN_THREADS) threads = CHAIN_THREADS;
+  if (d <= 256) {   // one step, or no cluster to be had
     size_t smem = sizeof(double2) * 2 * d;
-    state_chain_kernel<<<1, threads, smem, s>>>(n_steps, d, U, sU, psi, reorth_every, step_offset, traj);
+    state_chain_kernel<<<1, CHAIN_THREADS, smem, s>>>(n_steps, d, U, sU, psi, reorth_every, step_offset, traj);
     return check_launch("state_chain_kernel");
   }
   double* a = psi;
@@ -347,10 +380,9 @@ int launch_multi_chain(int nseg, int d, const ChainSeg* segs_dev, const double* 
   // clusters while all states' clusters run at once; beyond, one CTA per state keeps the
   // device as busy without the barriers
   const int C = d > 32 ? chain_cluster_size(d, nseg) : 1;
-  if (C > 1)
+  if (C > 1 || d <= 32)
     return launch_chain_cluster(C, nseg, d, 0, segs_dev, U, sU, nullptr, psi_dev, reorth_every, 0, nullptr, s);
-  const int threads = d <= 32 ? 256 : CHAIN_THREADS;
-  multi_chain_kernel<<<nseg, threads, sizeof(double2) * 2 * d, s>>>(d, segs_dev, U, sU, psi_dev, reorth_every);
+  multi_chain_kernel<<<nseg, CHAIN_THREADS, sizeof(double2) * 2 * d, s>>>(d, segs_dev, U, sU, psi_dev, reorth_every);
   return check_launch("multi_chain_kernel");
 }
 

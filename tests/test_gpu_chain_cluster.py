@@ -1,5 +1,5 @@
-"""The state chain on thread-block clusters (32 < d <= 256, csrc/propagate.cu) against plain
-matrix-vector steps: every cluster size's edges, trajectories, renormalisation."""
+"""The state chain on thread-block clusters (d <= 256, csrc/propagate.cu) against plain
+matrix-vector steps: one CTA and every cluster size's edges, trajectories, renormalisation."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ from paper_2411_09982_gb300 import magnus as M  # noqa: E402
 
 
 @pytest.mark.parametrize("reorth", [0, 3])
-@pytest.mark.parametrize("d", [33, 48, 49, 96, 97, 129, 193, 255, 256])
+@pytest.mark.parametrize("d", [1, 2, 7, 31, 32, 33, 48, 49, 64, 65, 96, 97, 129, 193, 255, 256])
 def test_chain_matches_matrix_vector_steps(d, reorth):
     rng = np.random.default_rng(d)
     N = 7
