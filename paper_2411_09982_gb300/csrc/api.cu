@@ -525,10 +525,37 @@ struct Engine {
     return MG_OK;
   }
   int timing_begin(int* idx) { return timing_mark(ctx, idx); }
+  // FP64 exponentials of real symmetric exponents from digits
+  bool real64() const { return digits64() && x_sym; }
   // real products on the lower triangle that degree m and sq squarings take
   static int real_products(int m, int sq) {
     const int kc = m / 2, ks = (m - 1) / 2, p = (kc + 1) / 2;
     return p + (kc > p) + (ks > p) + 1 + 2 * sq;
+  }
+  int expm_real64(int batch, const double* W, const double* tau, int m, int per_poly, int sq, const int* sq_dev,
+                  double* U) {
+    products += (long long)batch * (per_poly + sq);
+    const long long md = 2LL * d * d, half = (long long)d * d * batch;
+    double* mats[8];
+    const int slots[4] = {WS_P2, WS_P3, WS_Y, WS_R0};
+    for (int q = 0; q < 4; ++q) {
+      MG_TRY(ws(ctx, slots[q], md * batch, &mats[2 * q]));
+      mats[2 * q + 1] = mats[2 * q] + half;
+    }
+    MG_TRY(reserve(batch));
+    // two of the four digit buffers share the larger B slot
+    void* digs[4] = {abuf, bbuf[0], static_cast<char*>(bbuf[0]) + f64r_bytes(d, batch), bbuf[1]};
+    int e0 = -1, e1 = -1;
+    if (ctx->timing) MG_TRY(timing_begin(&e0));
+    MG_TRY(f64r_expm(d, batch, W, tau, m, sq, sq_dev, mats, digs, U, ctx->slot_ptr[WS_F64_SUMS], ctx->sms, ctx->status,
+                     ctx->stream, ctl()));
+    if (ctx->timing) {
+      MG_TRY(timing_begin(&e1));
+      ctx->ev_pending.emplace_back(e0, e1);
+      ctx->t_launches += 1;
+      ctx->t_flops += (double)d * d * (d + 1) * real_products(m, sq_dev ? 0 : sq) * batch;
+    }
+    return MG_OK;
   }
   // FP64 exponentials in one launch (expm_small.cu)
   bool small64() const { return prec == MG_PREC_FP64 && d <= expm_small_max_dim(); }
@@ -739,6 +766,10 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
     if (sU != md) return MG_EINVAL;
     return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, tc.s, nullptr, U);
   }
+  if (eng.real64()) {
+    if (sU != md) return MG_EINVAL;
+    return eng.expm_real64(batch, W, tau, tc.m, tc.products, tc.s, nullptr, U);
+  }
   // X = -i 2^{-s} W   (in place, into the engine's storage format)
   MG_TRY(eng.scale_x(batch, W, W, tc.s, nullptr, w_df));
   double *R, *Rn;
@@ -769,6 +800,7 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
                    const TaylorChoice& tc, int S, double* U, bool w_df) {
   PhaseRange range("expm");
   if (eng.small64()) return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, S, sq_dev, U);
+  if (eng.real64()) return eng.expm_real64(batch, W, tau, tc.m, tc.products, S, sq_dev, U);
   const long long md = mat_doubles(eng.d);
   MG_TRY(eng.scale_x(batch, W, W, 0, sq_dev, w_df));
   double *R, *Rn;

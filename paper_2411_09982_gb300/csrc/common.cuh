@@ -200,6 +200,12 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
               long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
               int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
 
+// FP64 exponentials of real symmetric exponents from digits (cosine and sine, real symmetric
+// products); see f64r_expm.
+size_t f64r_bytes(int d, int batch);
+int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int sq, const int* sq_dev, double* const* mats,
+              void* const* digs, double* U, void* scratch, int sms, int* status, cudaStream_t s, const SplitCtl& ctl0);
+
 // FP64 exponentials of small matrices (d <= expm_small_max_dim()), U_b = e^{-i tau_b}
 // exp(-i W_b) (tau may be null), in one launch; see expm_small.cu.  Degree m and block p as
 // Paterson-Stockmeyer takes them; sq_dev: per-item squaring counts, else sq; real_sym: every

@@ -7,25 +7,28 @@
 // whose products the tensor cores accumulate exactly (the error-free splitting of Ozaki,
 // Ogita, Oishi and Rump, Numerical Algorithms 59, 2012):
 //   * Every row of A (column of B) is scaled by the power of two 2^E that bounds it and
-//     rounded to 56-bit fixed point: an entry a becomes F = rint(a 2^{55 - E}), |F| < 2^55,
-//     and F = sum_{s<8} q_s 2^{7 (7 - s)} with balanced base-128 digits |q_s| <= 64, each
-//     exact in BF16 (stored as q_s 2^{-7 s}).  Entries of the row's own binade keep all 53
-//     bits of their mantissa.
-//   * Digit products q_s q_t with s + t <= 8 (43 of 64; the rest lie 2^-7 below the rounding
-//     of F) are summed by level l = s + t in FP32 TMEM accumulators.  A product is at most
-//     2^12, so (l + 1) K products stay below 2^24, an exact integer, while
-//     (l + 1) K <= 4096: the accumulators are drained into 64-bit integer registers every
-//     KSEG positions of K (1024 for levels 0..3, 576 for levels 4..7).  Level 8 shares level
-//     7's accumulator; their sum, 2^-49 below the leading digit product, is the only one
-//     that FP32 rounds (to 2^-7 of level 7's unit while it is below 2^17).
-//   * The two 64-bit sums (levels 0..3 and 4..8) are joined by one FP64 FMA, the product's
+//     rounded to 63-bit fixed point: an entry a becomes F = rint(a 2^{62 - E}), |F| < 2^62,
+//     and F = sum_{s<8} q_s 2^{8 (7 - s)} with balanced base-256 digits |q_s| <= 128 (the
+//     first at most 64), each exact in BF16 (stored as q_s 2^{-8 s}).  Entries down to 2^-9
+//     of the row's largest keep all 53 bits of their mantissa.
+//   * Digit products q_s q_t with s + t <= 7 (36 of 64) are summed by level l = s + t in FP32
+//     TMEM accumulators.  Their levels up to 5 have to stay exact integers below 2^24 (the
+//     rounding of level 6 and 7 weighs 2^-62 of the leading digit product and less), so the
+//     accumulators are drained into 64-bit integer registers every n K steps of 32: by
+//     Cauchy-Schwarz a level's sum over n steps is at most n sqrt(ea eb), ea and eb the
+//     largest digit energies (sums of q_s^2) of one K step in A's rows and B's columns, which
+//     the slicers record per item.  Full random digits give n = 12 and 18 (levels 0..3),
+//     whatever the operands 6 and 10 steps are exact, and most matrices of the exponential
+//     take one drain per sweep.
+//   * The two 64-bit sums (levels 0..3 and 4..7) are joined by one FP64 FMA, the product's
 //     only rounding beside that of F.
-// The error is about 2^-57 sqrt(K) of (largest entry of the row of A) x (rms entry of the
-// column of B) and the same with A and B exchanged: for the exponential's matrices no
-// larger than that of FP64 arithmetic, whose K roundings accumulate.  (Without level 8 the
-// dropped digit products weigh 2^-56 sqrt(K) of the largest entries on both sides, which
-// near-diagonal matrices show: 1.6e-14 of a row's norm at d = 729 against FP64's 2e-15.)  Operands that the scheme does not cover -- a NaN, an
-// infinity, a row or column whose largest entry lies outside 2^-400 .. 2^400 -- are marked
+// The error is about 2^-58 of (largest entry of the row of A) x (largest entry of the column
+// of B) beside the rounding of the result: below FP64 arithmetic's, whose K roundings
+// accumulate.  Whole evolutions against quad precision (relative 2-norm, here / FP64 pipe):
+// spin chain d = 64, six squarings per interval 2.1e-14 / 5.6e-14, four 4.4e-15 / 3.2e-14;
+// transmon chain d = 81 2.7e-14 / 1.1e-13; transmon-resonator d = 80 1.1e-12 / 1.6e-12.
+// (Base-128 digits, 56 bits, need fewer drains but gave 2.3e-14, 1.3e-14, 1.0e-13, 1.1e-12.)
+// Operands that the scheme does not cover -- a NaN, an infinity, a row or column whose largest entry lies outside 2^-400 .. 2^400 -- are marked
 // by the slicers; such an item is left to the FP64-pipe product, which is launched behind
 // and returns at once for all others.
 //
@@ -35,20 +38,20 @@
 //               in a ring of six.  Levels 0..3 need the digits 0..3 of A and B (two slots per
 //               K step), levels 4..7 all eight (four slots).
 //   warp 1      MMA issuer: M = 128, N = 128 (64 real, 64 imaginary columns), K = 16; four
-//               levels fill the 512 TMEM columns.  In the sweep of levels 4..8 the order
-//               (A 0..3, B 0..3), (A 0..3, B 4..7), (A 4..7, B 4..7), (A 4..7, B 0..3) frees
-//               two slots while 13 digit pairs are still to be multiplied, so a ring of 1.5 K
-//               steps keeps loads in flight.
+//               levels fill the 512 TMEM columns.  In the sweep of levels 4..7 the order
+//               (A 0..3, B 0..3), (A 0..3, B 4..7), (A 4..7, B 0..3) frees two slots while
+//               ten digit pairs are still to be multiplied, so a ring of 1.5 K steps keeps
+//               loads in flight.
 //   warps 2..9  drains: tcgen05.ld, float -> int, 64-bit accumulation in registers (64 sums
 //               per thread).  The sums of levels 4..7 wait in a per-CTA scratch (L2) while
 //               levels 0..3 are swept.  Conversion to FP64, scaling, addends and stores run
 //               while the next tile's MMAs are issued: the FP64 pipe (4 operations per output)
 //               is idle otherwise.
 // Measured (GB300, one product of a batch, slicing included): d = 729 2804 us on the FP64
-// pipe -> 110 us (28 TFLOP/s of the product's 8 d^3); d = 256 112 -> 8.3 us; d = 81 8.9 ->
-// 1.5 us.  At d = 729 the slicers take 12% (HBM-bound), the tensor pipe is active 67% of
-// the product's cycles: the rest goes to the drains (five per tile, ~4000 cycles of
-// float-to-int conversions each) and to operand delivery (single CTAs load 43 bytes per
+// pipe -> 109 us (28 TFLOP/s of the product's 8 d^3); d = 256 112 -> 8.8 us; d = 81 8.9 ->
+// 1.5 us.  At d = 729 the slicers take 12% (HBM-bound) and the tensor pipe is active about
+// two thirds of the product's cycles: the rest goes to the drains (~5000 cycles each,
+// float-to-int conversions above all) and to operand delivery (single CTAs load 43 bytes per
 // cycle and SM).
 // Every wait is bounded (SplitCtl::wait_ns, at most 4 s): a wait that gives up records
 // MG_DEV_TIMEOUT, the CTA's unfinished tiles become NaN, and it leaves once its own copies
@@ -70,8 +73,8 @@ constexpr int F8_SLOTS = 6;
 constexpr int F8_SLOT_BYTES = 4 * F8_BM * F8_BK * 2;
 constexpr int F8_THREADS = 320;
 constexpr int F8_EPI_WARPS = 8;
-constexpr int F8_SEG_LO = 18;           // K steps per drain of levels 4..7 (576 positions of K)
-constexpr int F8_SEG_HI = 32;           // and of levels 0..3 (1024)
+constexpr int F8_SEG_LO = 6;            // K steps per drain of levels 4..7 that are exact whatever the digits
+constexpr int F8_SEG_HI = 10;           // and of levels 0..3
 constexpr int F8_VALS = 64;             // sums per epilogue thread
 constexpr int F8_STAGE_BYTES = F8_EPI_WARPS * 32 * 8 * 16;   // epilogue staging: 32 rows x 8 columns per warp
 constexpr int F8_EXP_MAX = 400;
@@ -90,12 +93,13 @@ static F8Geom f8_geom(int d) {
   return g;
 }
 
-// operand buffer: digits of all items, then row (column) exponents, then the items' marks
+// operand buffer: digits of all items, then row (column) exponents, then the items' marks and
+// digit energies
 size_t f64d_a_bytes(int d, int batch) {
-  return ((size_t)f8_geom(d).a_elems * 2 + (size_t)d * 4 + 4) * batch;
+  return ((size_t)f8_geom(d).a_elems * 2 + (size_t)d * 4 + 12) * batch;
 }
 size_t f64d_b_bytes(int d, int batch) {
-  return ((size_t)f8_geom(d).b_elems * 2 + (size_t)d * 4 + 4) * batch;
+  return ((size_t)f8_geom(d).b_elems * 2 + (size_t)d * 4 + 12) * batch;
 }
 
 // ---------------------------------------------------------------------------
@@ -108,32 +112,67 @@ __device__ __forceinline__ int f8_exp(double a) {
 }
 __device__ __forceinline__ bool f8_marked(int E) { return E > F8_EXP_MAX || (E < -F8_EXP_MAX && E > -(1 << 28)); }
 
-constexpr unsigned long long F8_BIAS = 0x0102040810204081ull * 64;   // 64 in every base-128 position 0..8
-// F + bias for F = rint(a 2^{55 - E}): digit s is ((F + bias) >> 7 (7 - s)) mod 128 - 64, the
-// top one without the mod.  The fixed-point value is formed on the integer pipe.
+constexpr unsigned long long F8_BIAS = 0x8080808080808080ull;   // 128 in every base-256 position
+// F + bias for F = rint(a 2^{62 - E}), |F| < 2^62: digit s is byte 7 - s of the sum, less 128.
+// The fixed-point value is formed on the integer pipe.
 __device__ __forceinline__ unsigned long long f8_fixed(double a, int E) {
   const long long bits = __double_as_longlong(a);
   const int bexp = (int)((bits >> 52) & 0x7FF);
-  const int sh = bexp - 1075 + 55 - E;                       // <= 2
+  const int sh = bexp - 1075 + 62 - E;                       // <= 9
   unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  if (sh >= 0) m <<= min(sh, 2);
+  if (sh >= 0) m <<= min(sh, 9);
   else if (sh > -56) m = (m + (1ull << (-sh - 1))) >> -sh;
   else m = 0;
   if (bexp == 0) m = 0;                                      // zero (a subnormal is below any kept bit)
-  const unsigned long long f = bits < 0 ? 0ull - m : m;
-  return f + (F8_BIAS & 0x00FFFFFFFFFFFFFFull);
+  return (bits < 0 ? 0ull - m : m) + F8_BIAS;
 }
-// q_s 2^{-7 s} of a biased value as FP32 (exact): the field in the low mantissa bits of
-// 2^{23 - 7 s}, less (2^23 + 64) 2^{-7 s}
+// q_s 2^{-8 s} of a biased value as FP32 (exact): the byte in the low mantissa bits of
+// 2^{23 - 8 s}, less (2^23 + 128) 2^{-8 s}
 __device__ __forceinline__ float f8_digit(unsigned long long f, int s) {
-  uint32_t q = (uint32_t)(f >> (7 * (7 - s)));
-  q = s == 0 ? (q & 0xFFu) : (q & 0x7Fu);
-  const uint32_t magic = 0x4B000000u - ((uint32_t)(7 * s) << 23);
-  return __uint_as_float(magic | q) - __uint_as_float(magic | 64u);
+  const uint32_t q = (uint32_t)(f >> (8 * (7 - s))) & 0xFFu;
+  const uint32_t magic = 0x4B000000u - ((uint32_t)(8 * s) << 23);
+  return __uint_as_float(magic | q) - __uint_as_float(magic | 128u);
 }
 // BF16 pair (lo in the low half); the digits are exact in the high 16 bits of their FP32 form
 __device__ __forceinline__ uint32_t f8_pack(float lo, float hi) {
   return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+}
+
+// Digit energies, the bound on the level sums: sum of q_s^2 over s <= 5 (high half) and s <= 3
+// (low half) in units of 64, rounded up, so that the sum over one row's (column's) 32
+// positions of a K step fits 16 bits each.
+__device__ __forceinline__ uint32_t f8_energy(const unsigned long long (&f)[4]) {
+  int e3 = 0, e5 = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int hi = (int)((uint32_t)(f[q] >> 32) ^ 0x80808080u);             // digits 0..3 as signed bytes
+    const int lo = (int)(((uint32_t)f[q] ^ 0x80808080u) & 0xFFFF0000u);     // digits 4, 5
+    e3 = __dp4a(hi, hi, e3);
+    e5 = __dp4a(lo, lo, e5);
+  }
+  return ((uint32_t)(e3 + e5 + 63) >> 6 << 16) | ((uint32_t)(e3 + 63) >> 6);
+}
+// over the 8 lanes that share a row's K step, then the larger of both halves of two values
+__device__ __forceinline__ uint32_t f8_energy_step(uint32_t e) {
+  for (int o = 1; o < 8; o <<= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  return e;
+}
+__device__ __forceinline__ uint32_t f8_energy_max(uint32_t a, uint32_t b) { return __vmaxu2(a, b); }
+// the warp's largest into the item's two words (s <= 5, s <= 3)
+__device__ __forceinline__ void f8_energy_store(uint32_t e, uint32_t* item, int lane) {
+  for (int o = 16; o >= 8; o >>= 1) e = f8_energy_max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  if (lane == 0) {
+    if (item[0] < (e >> 16)) atomicMax(item, e >> 16);
+    if (item[1] < (e & 0xFFFFu)) atomicMax(item + 1, e & 0xFFFFu);
+  }
+}
+// K steps that keep every level sum of a segment below 2^24 by Cauchy-Schwarz, given the
+// largest energies of both operands' K steps: n sqrt(ea eb) <= 2^24 (0.1% below, for the
+// rounding of this expression)
+__device__ __forceinline__ int f8_seg(uint32_t ea, uint32_t eb, int least, int steps) {
+  const float e = (float)ea * (float)eb;   // in units of 64^2
+  const int n = e > 0.f ? (int)(fminf(261881.0f * rsqrtf(e), 4096.0f)) : steps;
+  return min(max(n, least), steps);
 }
 
 // A digits, one warp per row: row exponent, then 4 consecutive elements per lane and step.
@@ -141,7 +180,7 @@ __device__ __forceinline__ uint32_t f8_pack(float lo, float hi) {
 // entry written, 16 read).
 __global__ void __launch_bounds__(256)
 f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2, __nv_bfloat16* __restrict__ out,
-                    long long item_elems, int* __restrict__ ea, int* __restrict__ bad,
+                    long long item_elems, int* __restrict__ ea, int* __restrict__ bad, uint32_t* __restrict__ energy,
                     const int* __restrict__ item_sq, int sq_step) {
   const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y;
   if (row >= d) return;
@@ -162,7 +201,9 @@ f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2,
   }
   __nv_bfloat16* o = out + b * item_elems + (long long)row * Kp;
   const long long ds = (long long)d * Kp;
-  for (int k = 4 * lane; k < Kh; k += 128) {
+  uint32_t en = 0;
+  for (int k0 = 0; k0 < Kh; k0 += 128) {
+    const int k = k0 + 4 * lane;
     unsigned long long re[4], im[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -170,6 +211,8 @@ f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2,
       re[q] = f8_fixed(v.x, E);
       im[q] = f8_fixed(v.y, E);
     }
+    en = f8_energy_max(en, f8_energy_max(f8_energy_step(f8_energy(re)), f8_energy_step(f8_energy(im))));
+    if (k >= Kh) continue;
 #pragma unroll
     for (int s = 0; s < F8_L; ++s) {
       *reinterpret_cast<uint2*>(o + s * ds + k) =
@@ -178,6 +221,7 @@ f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2,
           make_uint2(f8_pack(f8_digit(im[0], s), f8_digit(im[1], s)), f8_pack(f8_digit(im[2], s), f8_digit(im[3], s)));
     }
   }
+  f8_energy_store(en, energy + 2 * b, lane);
 }
 
 // Column exponents (preset to byte 0x80): grid (ceil(d/64), ceil(d/64), batch), block 256.
@@ -207,7 +251,7 @@ f64d_col_exponent_kernel(int d, const double2* __restrict__ B, long long sB2, in
 template <bool ADJ>
 __global__ void __launch_bounds__(256)
 f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB2, __nv_bfloat16* __restrict__ out,
-                      long long item_elems, int* __restrict__ eb, int* __restrict__ bad,
+                      long long item_elems, int* __restrict__ eb, int* __restrict__ bad, uint32_t* __restrict__ energy,
                       const int* __restrict__ item_sq, int sq_step) {
   __shared__ double2 tile[32][65];
   __shared__ int ex[64];
@@ -225,9 +269,9 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
     tile[kk][c] = (k0 + kk < d && j0 + c < d) ? Bb[(long long)(k0 + kk) * d + j0 + c] : make_double2(0.0, 0.0);
   }
   __syncthreads();
-  for (int e = tid; e < 8 * 64; e += 256) {
+  uint32_t en = 0;
+  for (int e = tid; e < 8 * 64; e += 256) {   // 8 lanes per column
     const int g = e & 7, r = e >> 3, j = j0 + r, k = k0 + 4 * g;
-    if (j >= d) continue;
     const int E = ex[r];
     unsigned long long re[4], im[4];
 #pragma unroll
@@ -236,6 +280,8 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
       re[q] = f8_fixed(v.x, E);
       im[q] = f8_fixed(ADJ ? -v.y : v.y, E);
     }
+    en = f8_energy_max(en, f8_energy_max(f8_energy_step(f8_energy(re)), f8_energy_step(f8_energy(im))));
+    if (j >= d) continue;
     if constexpr (ADJ) {
       __nv_bfloat16* o = out + b * item_elems + (long long)j * Kp + k;
       const long long ds = (long long)d * Kp;
@@ -261,25 +307,117 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
       }
     }
   }
+  f8_energy_store(en, energy + 2 * b, tid & 31);
   // the exponents of all-zero columns stay preset; the product reads them as 0
+}
+
+// Row digits of a real symmetric matrix (both operands of its products are such rows), one
+// warp per row: entry k is X[k] + sz Z[k] (Z null: X[k]), or with CW the real part of a complex
+// matrix W times 2^{-sq} (an exact change of the row's exponent).  grid (ceil(d / 8), batch).
+// Entries are bounded (the exponential scales them to norm about 1); rows below 2^-400 are
+// rounded at that scale, far below anything the result holds.
+template <bool CW>
+__global__ void __launch_bounds__(256)
+f64r_slice_kernel(int d, int Kh, const double* __restrict__ X, const double* __restrict__ Z, double sz, long long sX,
+                  int sq, const int* __restrict__ sq_dev, __nv_bfloat16* __restrict__ out, long long item_elems,
+                  int* __restrict__ ex, uint32_t* __restrict__ energy, const int* __restrict__ item_sq, int sq_step) {
+  const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y;
+  if (row >= d) return;
+  if (item_sq && item_sq[b] <= sq_step) return;
+  const double* x = X + b * sX + (long long)row * d * (CW ? 2 : 1);
+  const double* z = Z ? Z + b * sX + (long long)row * d : nullptr;
+  auto load = [&](int k) {
+    if constexpr (CW) return x[2 * k];
+    else return z ? fma(sz, z[k], x[k]) : x[k];
+  };
+  int E = -(1 << 29);
+  for (int k = lane; k < d; k += 32) E = max(E, f8_exp(load(k)));
+  for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+  const int s = CW ? (sq_dev ? sq_dev[b] : sq) : 0;
+  if (E < -(1 << 28)) E = s;                 // all-zero row
+  E = max(E, s - F8_EXP_MAX);
+  if (lane == 0) ex[(long long)b * d + row] = E - s;
+  __nv_bfloat16* o = out + b * item_elems + (long long)row * Kh;
+  const long long ds = (long long)d * Kh;
+  uint32_t en = 0;
+  for (int k0 = 0; k0 < Kh; k0 += 128) {
+    const int k = k0 + 4 * lane;
+    unsigned long long f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f[q] = f8_fixed(k + q < d ? load(k + q) : 0.0, E);
+    en = f8_energy_max(en, f8_energy_step(f8_energy(f)));
+    if (k >= Kh) continue;
+#pragma unroll
+    for (int g = 0; g < F8_L; ++g)
+      *reinterpret_cast<uint2*>(o + g * ds + k) =
+          make_uint2(f8_pack(f8_digit(f[0], g), f8_digit(f[1], g)), f8_pack(f8_digit(f[2], g), f8_digit(f[3], g)));
+  }
+  f8_energy_store(en, energy + 2 * b, lane);
+}
+
+// Real symmetric matrices: two linear combinations of up to four matrices in one pass,
+// dst_o = sum_m coef[o][m] src_m + diag[o] I (dst_1 may be null).
+struct RealComb {
+  const double* src[4];
+  double coef[2][4], diag[2];
+  double* dst[2];
+  int n;
+};
+__global__ void __launch_bounds__(256) f64r_lincomb_kernel(int d, long long total, const __grid_constant__ RealComb a) {
+  const long long per = (long long)d * d;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+    const long long r = e % per;
+    const bool dg = r / d == r % d;
+    double v0 = dg ? a.diag[0] : 0.0, v1 = dg ? a.diag[1] : 0.0;
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (m < a.n) {
+        const double x = a.src[m][e];
+        v0 = fma(a.coef[0][m], x, v0);
+        v1 = fma(a.coef[1][m], x, v1);
+      }
+    if (a.dst[0]) a.dst[0][e] = v0;
+    if (a.dst[1]) a.dst[1][e] = v1;
+  }
+}
+
+// U_b = e^{-i tau_b} (C_b - i S_b); grid (x, batch)
+__global__ void __launch_bounds__(256)
+f64r_phase_kernel(long long per, const double* __restrict__ tau, const double* __restrict__ C,
+                  const double* __restrict__ S, double2* __restrict__ U) {
+  __shared__ double ph[2];
+  const long long o = blockIdx.y * per;
+  if (threadIdx.x == 0) {
+    ph[0] = 1.0;
+    ph[1] = 0.0;
+    if (tau) sincos(tau[blockIdx.y], &ph[1], &ph[0]);
+  }
+  __syncthreads();
+  const double cs = ph[0], sn = ph[1];
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per; e += (long long)gridDim.x * blockDim.x) {
+    const double c = C[o + e], s = S[o + e];
+    U[o + e] = make_double2(cs * c - sn * s, -(sn * c + cs * s));
+  }
 }
 
 // ---------------------------------------------------------------------------
 // product
 // ---------------------------------------------------------------------------
 struct F8Args {
-  int d, Kp, batch, ntn, ntm;
+  int d, Kp, batch, ntn, ntm;   // Kp: length of the K axis; per item ntm x ntn tiles
   const int* ea;
   const int* eb;
   const int* bad_a;
   const int* bad_b;
+  const uint32_t* en_a;       // per item: largest digit energies of a K step (f8_energy)
+  const uint32_t* en_b;
   double* C;
   long long sC;               // doubles
   const double* add_src[3];
   double add_coef[3];
   long long add_stride;       // doubles
   int add_n;
-  double diag;
+  double diag, scale;         // scale: real products only
   long long* scratch;         // per CTA: F8_VALS x 256 sums of levels 4..7
   int* status;
   const int* item_sq;
@@ -289,7 +427,7 @@ struct F8Args {
 };
 
 __device__ __forceinline__ bool f8_skip(const F8Args& p, int b) {
-  return (p.bad_a[b] | p.bad_b[b]) != 0 || (p.item_sq && p.item_sq[b] <= p.sq_step);
+  return (p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.item_sq && p.item_sq[b] <= p.sq_step);
 }
 
 // polls until the phase completes, the CTA aborts or the limit runs out
@@ -308,32 +446,50 @@ __device__ __forceinline__ double f8_to_double(long long x) {
 }
 
 // Drain of one accumulator set (levels l0 .. l0 + 3) into the thread's sums, in units of
-// 2^{-7 (l0 + 3)}.  With KSEG as above |G_l| 128 + |G_{l+1}| fits 32 bits for the integers
-// G_l = 2^{7 l} g_l.
+// 2^{-8 (l0 + 3)}, from the integers G_l = 2^{8 l} g_l.
+template <bool CPLX>
 __device__ __forceinline__ void f8_drain(uint32_t tbase, int l0, long long (&acc)[F8_VALS]) {
-  const float m0 = l0 ? 268435456.0f : 1.0f;   // 2^{7 l0}
-  const float m1 = m0 * 128.0f, m2 = m0 * 16384.0f, m3 = m0 * 2097152.0f;
+  const float m0 = l0 ? 4294967296.0f : 1.0f;   // 2^{8 l0}
+  const float m1 = m0 * 256.0f, m2 = m0 * 65536.0f, m3 = m0 * 16777216.0f;
 #pragma unroll
   for (int c = 0; c < F8_VALS; c += 8) {
-    // values 0..31: real parts of the thread's 32 columns, 32..63: imaginary parts
-    const uint32_t col = tbase + (c < 32 ? c : F8_BN + c - 32);
+    // complex: values 0..31 are the real parts of the thread's 32 columns, 32..63 the imaginary
+    // parts; real: 64 columns
+    const uint32_t col = tbase + (CPLX && c >= 32 ? F8_BN + c - 32 : c);
     uint32_t g[4][8];
 #pragma unroll
     for (int l = 0; l < 4; ++l) tmem_ld8(col + l * 128, g[l]);
     tmem_wait_ld();
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
-      const int i01 = __float2int_rn(__uint_as_float(g[0][v]) * m0) * 128 +
-                      __float2int_rn(__uint_as_float(g[1][v]) * m1);
-      const int i23 = __float2int_rn(__uint_as_float(g[2][v]) * m2) * 128 +
-                      __float2int_rn(__uint_as_float(g[3][v]) * m3);
-      acc[c + v] += (long long)i01 * 16384 + i23;
+      acc[c + v] += (long long)__float2int_rn(__uint_as_float(g[0][v]) * m0) * 16777216 +
+                    (long long)__float2int_rn(__uint_as_float(g[1][v]) * m1) * 65536;
+      acc[c + v] += (long long)__float2int_rn(__uint_as_float(g[2][v]) * m2) * 256 +
+                    __float2int_rn(__uint_as_float(g[3][v]) * m3);
     }
   }
 }
 
 constexpr uint32_t kF8Idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
+// tile `rem` of an item: row by row, or (SYM: real symmetric products) the lower triangle
+template <bool CPLX>
+__device__ __forceinline__ void f8_tile(const F8Args& p, int rem, int& mt, int& nt) {
+  if constexpr (CPLX) {
+    mt = rem / p.ntn;
+    nt = rem % p.ntn;
+  } else {
+    mt = 0;
+    while ((mt + 1) * (mt + 2) / 2 <= rem) ++mt;   // at most 32 row tiles
+    nt = rem - mt * (mt + 1) / 2;
+  }
+}
+
+// CPLX: 128 x 64 complex tiles as described above.  Otherwise products of commuting real
+// symmetric matrices (polynomials in one matrix): both operands are row digits, tiles are
+// 128 x 128 real entries on and below the diagonal, and every entry is written on both sides
+// of it; addends are symmetric too.
+template <bool CPLX>
 __global__ void __launch_bounds__(F8_THREADS, 1)
 f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ F8Args p) {
@@ -372,9 +528,13 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int steps = p.Kp / F8_BK, half = steps / 2;
-  const int per_item = p.ntn * p.ntm;
+  const int per_item = CPLX ? p.ntn * p.ntm : p.ntm * (p.ntm + 1) / 2;
   const long long tiles = (long long)per_item * p.batch;
-  const int nseg[2] = {(steps + F8_SEG_LO - 1) / F8_SEG_LO, (steps + F8_SEG_HI - 1) / F8_SEG_HI};   // levels 4..7, 0..3
+  // drains of an item's sweep (0: levels 4..7, 1: levels 0..3)
+  auto segments = [&](int b, int sweep) {
+    const int n = f8_seg(p.en_a[2 * b + sweep], p.en_b[2 * b + sweep], sweep == 0 ? F8_SEG_LO : F8_SEG_HI, steps);
+    return (steps + n - 1) / n;
+  };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -382,7 +542,9 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       long long n = 0;   // slots filled
       bool ok = true;
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        const int b = (int)(t / per_item), rem = (int)(t % per_item), mt = rem / p.ntn, nt = rem % p.ntn;
+        const int b = (int)(t / per_item);
+        int mt, nt;
+        f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         if (f8_skip(p, b)) continue;
         for (int sweep = 0; sweep < 2 && ok; ++sweep) {
           const int per_step = sweep == 0 ? 4 : 2;
@@ -399,6 +561,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               unsigned char* dst = smem + s * F8_SLOT_BYTES;
               if (q == 0 || q == 3)
                 tma_load_4d(dst, &tmA, &full[s], st * F8_BK, mt * F8_BM, q == 0 ? 0 : 4, b);
+              else if constexpr (!CPLX)
+                tma_load_4d(dst, &tmB, &full[s], st * F8_BK, nt * F8_BM, q == 1 ? 0 : 4, b);
               else
                 tma_load_5d(dst, &tmB, &full[s], (imag ? st - half : st) * F8_BK, nt * F8_BN, imag ? 0 : 1,
                             q == 1 ? 0 : 4, b);
@@ -426,9 +590,10 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       uint32_t set = 0;   // accumulator sets begun
       bool ok = !p.stall || f8_wait(mmadone, 0, p.wait_ns, abort_flag);
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        if (f8_skip(p, (int)(t / per_item))) continue;
+        const int b = (int)(t / per_item);
+        if (f8_skip(p, b)) continue;
         for (int sweep = 0; sweep < 2 && ok; ++sweep) {
-          const int ns = nseg[sweep];
+          const int ns = segments(b, sweep);
           for (int sg = 0; sg < ns && ok; ++sg) {
             const int st0 = (int)((long long)steps * sg / ns), st1 = (int)((long long)steps * (sg + 1) / ns);
             if (!f8_wait(accempty, (set & 1) ^ 1u, p.wait_ns, abort_flag)) { ok = false; break; }
@@ -450,9 +615,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                   for (int s = 0; s < 4; ++s)
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                      int l = s0 + s + t0 + u;
+                      const int l = s0 + s + t0 + u;
                       if (l < lmin || l > lmax) continue;
-                      l = min(l, lmin + 3);   // level 8 with level 7
                       const uint64_t ad = sw64_kmajor_desc(abase + s * 8192 + kk * 32);
                       const uint64_t bd = sw64_kmajor_desc(bbase + u * 8192 + kk * 32);
                       tc_mma_bf16(tmem + (l & 3) * 128, ad, bd, kF8Idesc, first[l & 3] ? 0u : 1u);
@@ -463,16 +627,15 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               if (!ready(0) || !ready(1)) { ok = false; break; }
               tc_fence_after();
               if (sweep == 0) {
-                group(sa[0], sa[1], 0, 0, 4, 8, first);
+                group(sa[0], sa[1], 0, 0, 4, 7, first);
                 if (!ready(2)) { ok = false; break; }
                 tc_fence_after();
-                group(sa[0], sa[2], 0, 4, 4, 8, first);
+                group(sa[0], sa[2], 0, 4, 4, 7, first);
                 tc_commit(&empty[n % F8_SLOTS]);
+                tc_commit(&empty[(n + 2) % F8_SLOTS]);
                 if (!ready(3)) { ok = false; break; }
                 tc_fence_after();
-                group(sa[3], sa[2], 4, 4, 4, 8, first);
-                tc_commit(&empty[(n + 2) % F8_SLOTS]);
-                group(sa[3], sa[1], 4, 0, 4, 8, first);
+                group(sa[3], sa[1], 4, 0, 4, 7, first);
                 tc_commit(&empty[(n + 1) % F8_SLOTS]);
                 tc_commit(&empty[(n + 3) % F8_SLOTS]);
                 n += 4;
@@ -502,7 +665,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
     const int q = warp & 3;                    // TMEM lane quarter of this warp
-    const int c0 = ((warp - 2) >> 2) * 32;     // first of its 32 complex columns
+    constexpr int WC = CPLX ? 32 : 64;         // columns per warp
+    const int c0 = ((warp - 2) >> 2) * WC;
     const int et = threadIdx.x - 64;
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + c0;
     long long* scratch = p.scratch + (long long)blockIdx.x * F8_VALS * 256 + et;
@@ -511,21 +675,25 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     bool ok = true;
     long long t = blockIdx.x;
     for (; t < tiles; t += gridDim.x) {
-      const int b = (int)(t / per_item), rem = (int)(t % per_item), mt = rem / p.ntn, nt = rem % p.ntn;
+      const int b = (int)(t / per_item);
+      int mt, nt;
+      f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
       if (f8_skip(p, b)) continue;
-      const int row0 = mt * F8_BM + q * 32, col0 = nt * F8_BN + c0;
-      const bool live = row0 < p.d && col0 < p.d;   // uniform over the warp
+      const int row0 = mt * F8_BM + q * 32, col0 = nt * 2 * WC + c0;
+      // uniform over the warp; a real tile's columns right of all its rows are not needed
+      const bool live = row0 < p.d && col0 < p.d && (CPLX || col0 <= row0 + 31);
       long long acc[F8_VALS];
       for (int sweep = 0; sweep < 2 && ok; ++sweep) {
 #pragma unroll
         for (int v = 0; v < F8_VALS; ++v) acc[v] = 0;
-        for (int sg = 0; sg < nseg[sweep]; ++sg) {
+        const int ns = segments(b, sweep);
+        for (int sg = 0; sg < ns; ++sg) {
           bool got = true;
           if (lane == 0) got = f8_wait(accfull, set & 1, p.wait_ns, abort_flag);
           got = __shfl_sync(0xffffffffu, (int)got, 0) != 0;
           if (!got) { ok = false; break; }
           tc_fence_after();
-          if (live) f8_drain(tbase, sweep == 0 ? 4 : 0, acc);
+          if (live) f8_drain<CPLX>(tbase, sweep == 0 ? 4 : 0, acc);
           tc_fence_before();
           __syncwarp();
           if (lane == 0)
@@ -541,6 +709,46 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (!live) continue;
       const int row = row0 + lane;
       const int Ea = row < p.d ? p.ea[(long long)b * p.d + row] : 0;
+      if constexpr (!CPLX) {
+        // entry (row, col) goes to both sides of the diagonal: (col, row) straight from the
+        // registers (lanes are consecutive rows), (row, col) through the warp's staging
+        double* Cr = p.C + b * p.sC;
+        double* stg8 = reinterpret_cast<double*>(stg);
+        const int* ebp = p.eb + (long long)b * p.d;
+#pragma unroll
+        for (int c = 0; c < F8_VALS; c += 8) {
+          if (col0 + c < p.d && col0 + c <= row0 + 31) {
+            long long lo[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) lo[v] = scratch[(c + v) * 256];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+              const int col = col0 + c + v;
+              const int k = Ea + (col < p.d ? ebp[col] : 0) - 64;
+              double x = fma(f8_to_double(acc[c + v]), 268435456.0, f8_to_double(lo[v] >> 4)) *
+                         __hiloint2double((k + 1023) << 20, 0);
+              if (row < p.d && col <= row) {
+                const long long off = (long long)col * p.d + row;
+#pragma unroll
+                for (int m = 0; m < 3; ++m)
+                  if (m < p.add_n) x = fma(p.add_coef[m], p.add_src[m][b * p.add_stride + off], x);
+                if (col == row) x += p.diag;
+                x *= p.scale;
+                Cr[off] = x;
+              }
+              stg8[lane * 8 + (v ^ (lane & 7))] = x;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = i * 4 + (lane >> 3), cc = lane & 7;
+              const int grow = row0 + r, gcol = col0 + c + cc;
+              if (grow < p.d && gcol < grow) Cr[(long long)grow * p.d + gcol] = stg8[r * 8 + (cc ^ (r & 7))];
+            }
+            __syncwarp();
+          }
+        }
+      } else {
       int Eb = col0 + lane < p.d ? p.eb[(long long)b * p.d + col0 + lane] : 0;
       if (Eb < -(1 << 28)) Eb = 0;   // all-zero column
       const double2* addp[3];
@@ -559,11 +767,11 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
 #pragma unroll
           for (int v = 0; v < 8; ++v) {
-            // the value is T 2^{Ea + Eb - 61}, T = hi 2^28 + lo in units of 2^-49
-            const int k = Ea + __shfl_sync(0xffffffffu, Eb, c + v) - 61;
+            // the value is T 2^{Ea + Eb - 64}, T = hi 2^28 + lo / 2^4 in units of 2^-52
+            const int k = Ea + __shfl_sync(0xffffffffu, Eb, c + v) - 64;
             const double sc = __hiloint2double((k + 1023) << 20, 0);
-            const double re = fma(f8_to_double(acc[c + v]), 268435456.0, f8_to_double(lre[v])) * sc;
-            const double im = fma(f8_to_double(acc[32 + c + v]), 268435456.0, f8_to_double(lim[v])) * sc;
+            const double re = fma(f8_to_double(acc[c + v]), 268435456.0, f8_to_double(lre[v] >> 4)) * sc;
+            const double im = fma(f8_to_double(acc[32 + c + v]), 268435456.0, f8_to_double(lim[v] >> 4)) * sc;
             stg[lane * 8 + (v ^ (lane & 7))] = make_double2(re, im);
           }
           __syncwarp();
@@ -588,6 +796,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           __syncwarp();
         }
       }
+      }
     }
     if (!ok) {
       if (lane == 0) {
@@ -597,11 +806,16 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       // the tiles this CTA leaves unfinished are not left looking like a result
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
       for (; t < tiles; t += gridDim.x) {
-        const int b = (int)(t / per_item), rem = (int)(t % per_item), mt = rem / p.ntn, nt = rem % p.ntn;
+        const int b = (int)(t / per_item);
+        int mt, nt;
+        f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         const int row = mt * F8_BM + q * 32 + lane;
         if (f8_skip(p, b) || row >= p.d) continue;
-        for (int c = nt * F8_BN + c0; c < min(p.d, nt * F8_BN + c0 + 32); ++c)
-          reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
+        const int n0 = nt * 2 * WC + c0;
+        for (int c = n0; c < min(p.d, n0 + WC); ++c) {
+          if constexpr (CPLX) reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
+          else p.C[b * p.sC + (long long)row * p.d + c] = p.C[b * p.sC + (long long)c * p.d + row] = nan;
+        }
       }
     }
     tc_fence_before();
@@ -622,12 +836,14 @@ struct F8Buf {
   __nv_bfloat16* dig;
   int* e;
   int* bad;
+  uint32_t* energy;
 };
 static F8Buf f8_buf(void* buf, long long elems, int d, int batch) {
   F8Buf r;
   r.dig = reinterpret_cast<__nv_bfloat16*>(buf);
   r.e = reinterpret_cast<int*>(r.dig + elems * batch);
   r.bad = r.e + (long long)d * batch;
+  r.energy = reinterpret_cast<uint32_t*>(r.bad + batch);
   return r;
 }
 
@@ -638,18 +854,18 @@ int f64d_slice_a(int d, int batch, const double* A, long long sA, int opA, void*
   const F8Buf o = f8_buf(buf, g.a_elems, d, batch);
   const double2* A2 = reinterpret_cast<const double2*>(A);
   if (opA == 0) {
-    MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, sizeof(int) * (size_t)batch, s));
+    MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, 3 * sizeof(int) * (size_t)batch, s));
     f64d_slice_a_kernel<<<dim3(ceil_div(d, 8), batch), 256, 0, s>>>(d, g.Kp, A2, sA / 2, o.dig, g.a_elems, o.e, o.bad,
-                                                                    ctl.item_sq, ctl.sq_step);
+                                                                    o.energy, ctl.item_sq, ctl.sq_step);
     return check_launch("f64d_slice_a_kernel");
   }
   MG_CUDA_TRY(cudaMemsetAsync(o.e, 0x80, sizeof(int) * (size_t)d * batch, s));
-  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, sizeof(int) * (size_t)batch, s));
+  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, 3 * sizeof(int) * (size_t)batch, s));
   f64d_col_exponent_kernel<<<dim3(ceil_div(d, 64), ceil_div(d, 64), batch), 256, 0, s>>>(d, A2, sA / 2, o.e,
                                                                                           ctl.item_sq, ctl.sq_step);
   MG_TRY(check_launch("f64d_col_exponent_kernel"));
   f64d_slice_col_kernel<true><<<dim3(ceil_div(d, 64), g.Kh / 32, batch), 256, 0, s>>>(
-      d, g.Kp, A2, sA / 2, o.dig, g.a_elems, o.e, o.bad, ctl.item_sq, ctl.sq_step);
+      d, g.Kp, A2, sA / 2, o.dig, g.a_elems, o.e, o.bad, o.energy, ctl.item_sq, ctl.sq_step);
   return check_launch("f64d_slice_col_kernel");
 }
 
@@ -659,12 +875,12 @@ int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cud
   const F8Buf o = f8_buf(buf, g.b_elems, d, batch);
   const double2* B2 = reinterpret_cast<const double2*>(B);
   MG_CUDA_TRY(cudaMemsetAsync(o.e, 0x80, sizeof(int) * (size_t)d * batch, s));
-  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, sizeof(int) * (size_t)batch, s));
+  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, 3 * sizeof(int) * (size_t)batch, s));
   f64d_col_exponent_kernel<<<dim3(ceil_div(d, 64), ceil_div(d, 64), batch), 256, 0, s>>>(d, B2, sB / 2, o.e,
                                                                                           ctl.item_sq, ctl.sq_step);
   MG_TRY(check_launch("f64d_col_exponent_kernel"));
   f64d_slice_col_kernel<false><<<dim3(ceil_div(d, 64), g.Kh / 32, batch), 256, 0, s>>>(
-      d, g.Kp, B2, sB / 2, o.dig, g.b_elems, o.e, o.bad, ctl.item_sq, ctl.sq_step);
+      d, g.Kp, B2, sB / 2, o.dig, g.b_elems, o.e, o.bad, o.energy, ctl.item_sq, ctl.sq_step);
   return check_launch("f64d_slice_col_kernel");
 }
 
@@ -693,6 +909,8 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   p.eb = b.e;
   p.bad_a = a.bad;
   p.bad_b = b.bad;
+  p.en_a = a.energy;
+  p.en_b = b.energy;
   p.C = C;
   p.sC = sC;
   p.add_n = add.n;
@@ -708,14 +926,158 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   const long long tiles = (long long)p.ntn * p.ntm * batch;
   const int grid = (int)std::min<long long>(tiles, sms);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
-  MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel), (int)smem));
-  f64d_gemm_kernel<<<grid, F8_THREADS, smem, s>>>(ma, mb, p);
+  MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<true>), (int)smem));
+  f64d_gemm_kernel<true><<<grid, F8_THREADS, smem, s>>>(ma, mb, p);
   MG_TRY(check_launch("f64d_gemm_kernel"));
   // items the slicers marked (usually none: the launch returns at once)
   AddTerms rest = add;
   rest.item_sq = ctl.item_sq;
   rest.sq_step = ctl.sq_step;
   return launch_cgemm_f64_marked(batch, d, A, sA, opA, B, sB, C, sC, rest, a.bad, b.bad, sms, s);
+}
+
+// ---------------------------------------------------------------------------
+// exponentials of real symmetric exponents
+// ---------------------------------------------------------------------------
+static long long f64r_elems(int d) { return (long long)F8_L * d * ceil_div(d, F8_BK) * F8_BK; }
+size_t f64r_bytes(int d, int batch) {
+  return (((size_t)f64r_elems(d) * 2 + (size_t)d * 4 + 8) * batch + 255) / 256 * 256;
+}
+
+// U_b = e^{-i tau_b} (cos A_b - i sin A_b)^(2^s) with A_b = 2^{-s} W_b, W_b = Hbar_b - tau_b I
+// real and symmetric (held as complex).  The degree-m Taylor polynomial of exp(-i A) splits
+// exactly into C = sum (-1)^k Y^k / (2k)! and S = A sum (-1)^k Y^k / (2k+1)!, Y = A^2; powers up
+// to Y^p with 2 p >= m / 2 leave one product to each series, and a squaring takes two,
+// C' = (C + S)(C - S) and S' = 2 S C.  All are symmetric: d^2 (d + 1) flops a product against
+// 8 d^3 of the complex form (degree 16: 7 + 2 s such products against 6 + s).  U(T) of 20
+// intervals of the d = 729 chain (s = 3): 22.5 ms with complex products from digits, 9.7 ms so.
+// mats: eight d x d real matrices per item (Y1..Y4, T1, T2, C, S), digs: four digit buffers of
+// f64r_bytes.  sq_dev: per-item squaring counts (at most sq), else sq for every item.
+int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int sq, const int* sq_dev, double* const* mats,
+              void* const* digs, double* U, void* scratch, int sms, int* status, cudaStream_t s, const SplitCtl& ctl0) {
+  if (batch <= 0) return MG_OK;
+  if (batch > 65535) return MG_EUNSUPPORTED;
+  const int Kh = ceil_div(d, F8_BK) * F8_BK;
+  const long long elems = f64r_elems(d), dd = (long long)d * d;
+  SplitCtl ctl = ctl0;
+  ctl.item_sq = nullptr;
+  struct Dig {
+    __nv_bfloat16* dig;
+    int* e;
+    uint32_t* energy;   // largest over the matrices that pass through the buffer
+    CUtensorMap map;
+  } D[4];
+  for (int q = 0; q < 4; ++q) {
+    D[q].dig = reinterpret_cast<__nv_bfloat16*>(digs[q]);
+    D[q].e = reinterpret_cast<int*>(D[q].dig + elems * batch);
+    D[q].energy = reinterpret_cast<uint32_t*>(D[q].e + (long long)d * batch);
+    MG_CUDA_TRY(cudaMemsetAsync(D[q].energy, 0, 2 * sizeof(uint32_t) * (size_t)batch, s));
+    MG_TRY(make_digit_map(&D[q].map, D[q].dig, Kh, d, d, F8_L, batch, F8_BK, F8_BM, 4));
+  }
+  auto slice = [&](int q, const double* X, const double* Z, double sz) {
+    f64r_slice_kernel<false><<<dim3(ceil_div(d, 8), batch), 256, 0, s>>>(d, Kh, X, Z, sz, dd, 0, nullptr, D[q].dig, elems,
+                                                                         D[q].e, D[q].energy, ctl.item_sq, ctl.sq_step);
+    return check_launch("f64r_slice_kernel");
+  };
+  const int ntm = ceil_div(d, F8_BM);
+  const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
+  MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<false>), (int)smem));
+  // dst = scale (D[x] D[y] + sum_m coef_m src_m + diag I)
+  auto mul = [&](int x, int y, double* dst, int n, const double* const* src, const double* coef, double diag,
+                 double scale) {
+    F8Args p{};
+    p.d = d;
+    p.Kp = Kh;
+    p.batch = batch;
+    p.ntn = p.ntm = ntm;
+    p.ea = D[x].e;
+    p.eb = D[y].e;
+    p.en_a = D[x].energy;
+    p.en_b = D[y].energy;
+    p.C = dst;
+    p.sC = dd;
+    p.add_n = n;
+    for (int q = 0; q < n; ++q) { p.add_src[q] = src[q]; p.add_coef[q] = coef[q]; }
+    p.add_stride = dd;
+    p.diag = diag;
+    p.scale = scale;
+    p.scratch = reinterpret_cast<long long*>(scratch);
+    p.status = status;
+    p.item_sq = ctl.item_sq;
+    p.sq_step = ctl.sq_step;
+    p.stall = ctl.stall;
+    p.wait_ns = std::min<unsigned long long>(ctl.wait_ns, 4000000000ull);
+    const long long tiles = (long long)ntm * (ntm + 1) / 2 * batch;
+    f64d_gemm_kernel<false><<<(int)std::min<long long>(tiles, sms), F8_THREADS, smem, s>>>(D[x].map, D[y].map, p);
+    return check_launch("f64d_gemm_kernel (real)");
+  };
+  double f[18], cc[9], ss[9];
+  f[0] = 1.0;
+  for (int j = 1; j < 18; ++j) f[j] = f[j - 1] / j;
+  const int kc = m / 2, ks = (m - 1) / 2, p = (kc + 1) / 2;
+  for (int k = 0; k < 9; ++k) {
+    cc[k] = k <= kc ? ((k & 1) ? -f[2 * k] : f[2 * k]) : 0.0;
+    ss[k] = k <= ks ? ((k & 1) ? -f[2 * k + 1] : f[2 * k + 1]) : 0.0;
+  }
+  double* const* Y = mats;   // Y[q - 1] = Y^q
+  double *T1 = mats[4], *T2 = mats[5], *C = mats[6], *S = mats[7];
+  const bool hc = kc > p, hs = ks > p;
+  // D0: A; D1: Y, then the high part's digits; D2: Y^2, then Y^p; D3: sine's sum
+  f64r_slice_kernel<true><<<dim3(ceil_div(d, 8), batch), 256, 0, s>>>(d, Kh, W, nullptr, 0.0, 2 * dd, sq, sq_dev, D[0].dig,
+                                                                      elems, D[0].e, D[0].energy, nullptr, 0);
+  MG_TRY(check_launch("f64r_slice_kernel"));
+  MG_TRY(mul(0, 0, Y[0], 0, nullptr, nullptr, 0.0, 1.0));
+  int dp = 1;   // digits of Y^p
+  if (p >= 2 || hc || hs) MG_TRY(slice(1, Y[0], nullptr, 0.0));
+  if (p >= 2) {
+    MG_TRY(mul(1, 1, Y[1], 0, nullptr, nullptr, 0.0, 1.0));
+    MG_TRY(slice(2, Y[1], nullptr, 0.0));
+    dp = 2;
+  }
+  if (p >= 3) MG_TRY(mul(2, 1, Y[2], 0, nullptr, nullptr, 0.0, 1.0));
+  if (p >= 4) MG_TRY(mul(2, 2, Y[3], 0, nullptr, nullptr, 0.0, 1.0));
+  if (p >= 3) MG_TRY(slice(2, Y[p - 1], nullptr, 0.0));
+  RealComb a{};
+  a.n = p;
+  for (int q = 0; q < p; ++q) {
+    a.src[q] = Y[q];
+    a.coef[0][q] = hc ? (p + 1 + q <= kc ? cc[p + 1 + q] : 0.0) : cc[1 + q];
+    a.coef[1][q] = hs ? (p + 1 + q <= ks ? ss[p + 1 + q] : 0.0) : ss[1 + q];
+  }
+  a.diag[0] = hc ? cc[p] : cc[0];
+  a.diag[1] = hs ? ss[p] : ss[0];
+  a.dst[0] = hc ? T1 : C;
+  a.dst[1] = T2;   // sine's high part, or its whole sum
+  const long long total = dd * batch;
+  f64r_lincomb_kernel<<<(int)std::min<long long>((total + 255) / 256, (long long)sms * 16), 256, 0, s>>>(d, total, a);
+  MG_TRY(check_launch("f64r_lincomb_kernel"));
+  const double* low[3] = {Y[0], Y[1], Y[2]};
+  const int hd = dp == 1 ? 3 : 1;   // where the high part's digits go
+  if (hc) {
+    MG_TRY(slice(hd, T1, nullptr, 0.0));
+    MG_TRY(mul(hd, dp, C, p - 1, low, cc + 1, cc[0], 1.0));
+  }
+  double* sine = T2;
+  if (hs) {
+    MG_TRY(slice(hd, T2, nullptr, 0.0));
+    MG_TRY(mul(hd, dp, S, p - 1, low, ss + 1, ss[0], 1.0));
+    sine = S;
+  }
+  MG_TRY(slice(3, sine, nullptr, 0.0));
+  MG_TRY(mul(0, 3, S, 0, nullptr, nullptr, 0.0, 1.0));   // sin = A (sum)
+  for (int k = 0; k < sq; ++k) {
+    ctl.item_sq = sq_dev;   // items whose count is reached keep their matrices
+    ctl.sq_step = k;
+    MG_TRY(slice(0, C, S, 1.0));
+    MG_TRY(slice(1, C, S, -1.0));
+    MG_TRY(slice(2, S, nullptr, 0.0));
+    MG_TRY(slice(3, C, nullptr, 0.0));
+    MG_TRY(mul(0, 1, C, 0, nullptr, nullptr, 0.0, 1.0));
+    MG_TRY(mul(2, 3, S, 0, nullptr, nullptr, 0.0, 2.0));
+  }
+  f64r_phase_kernel<<<dim3((unsigned)std::min<long long>((dd + 1023) / 1024, 64), batch), 256, 0, s>>>(
+      dd, tau, C, S, reinterpret_cast<double2*>(U));
+  return check_launch("f64r_phase_kernel");
 }
 
 }  // namespace mg

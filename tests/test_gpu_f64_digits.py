@@ -1,10 +1,10 @@
 """FP64 products from digits on the tensor cores (csrc/gemm_f64_digits.cu).
 
 A two-interval propagator product U_1 U_0 (mg_propagate) is one such product from d = 33
-on.  It is held to the bound of its arithmetic against extended precision: every entry of
-a row (column) is rounded to 2^-56 of the power of two above its largest entry, digit
-products of level 9 and up (6 x 2^12 x 2^-63 of the scaled unit and their tail) are
-dropped, level 7 is rounded to its own unit, and the result is rounded to FP64.
+on.  It is held, against extended precision, to the bound of 56-bit operands (every entry
+of a row or column rounded to 2^-56 of the power of two above its largest entry, digit
+products of level 9 and up dropped, the last level rounded to its own unit, the result
+rounded to FP64); the eight base-256 digits hold 63.
 """
 import numpy as np
 import pytest
@@ -42,6 +42,9 @@ def matrices(kind, d, rng):
     if kind == "largest_digits":   # every digit of every entry at its largest: the exactness bound's worst case
         x = (127 / 128) * (1 - 2.0 ** -53)
         return np.full((d, d), x * (1 + 1j)), np.full((d, d), x * (1 - 1j))
+    if kind == "largest_bytes":    # the same in base 256: 63, 127, 127, ... in units of 2^-6
+        x = (63 + 127 / 255) / 64
+        return np.full((d, d), x * (1 + 1j)), np.full((d, d), x * (1 - 1j))
     if kind == "scaled":           # rows of A and columns of B 2^-120 .. 2^120
         s = 2.0 ** rng.integers(-120, 121, size=d)
         return s[:, None] * g(), g() * s[None, :]
@@ -52,7 +55,7 @@ def matrices(kind, d, rng):
     return z, w
 
 
-@pytest.mark.parametrize("kind", ["gauss", "near_identity", "largest_digits", "scaled", "sparse"])
+@pytest.mark.parametrize("kind", ["gauss", "near_identity", "largest_digits", "largest_bytes", "scaled", "sparse"])
 @pytest.mark.parametrize("d", [33, 64, 65, 127, 129, 200, 600])
 def test_product_within_its_bound(d, kind):
     rng = np.random.default_rng(d)
@@ -119,5 +122,56 @@ def test_bounded_wait_runs_out_and_context_recovers():
         ref = (V * np.exp(-1j * lam)) @ V.conj().T
         assert np.abs(out.cpu().numpy() - ref).max() <= 1e-11
         plan.close()
+    finally:
+        ctx.close()
+
+
+def symmetric(rng, d, norm):
+    A = rng.normal(size=(d, d))
+    A = A + A.T
+    A *= norm / np.abs(A - np.trace(A) / d * np.eye(d)).sum(0).max()
+    return A.astype(np.complex128)
+
+
+def exact_exp(A):
+    lam, V = np.linalg.eigh(A.real)
+    return (V * np.exp(-1j * lam)) @ V.T
+
+
+@pytest.mark.parametrize("d", [33, 64, 97, 128, 129, 257, 400])
+def test_real_symmetric_exponentials(d):
+    """Cosine and sine form over every Taylor degree (norms 1e-9 .. 30: degrees 2 to 16, squarings)."""
+    rng = np.random.default_rng(d)
+    ctx = M.Context(0)
+    try:
+        for norm in (1e-9, 1e-5, 1e-2, 0.08, 0.3, 0.7, 3.0, 30.0):
+            A = symmetric(rng, d, norm)
+            plan = M.Plan(ctx, torch.from_numpy(A).cuda(), None, M.MG_PREC_FP64)
+            plan.set_controls(1, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((1, 1, 0), dtype=torch.float64))
+            out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+            rep = plan.evolve(M.MG_OUT_PROPAGATOR, None, out)
+            # ~20 products of d-term sums, their errors doubled by every squaring (2^s <= 4 norm)
+            assert np.abs(out.cpu().numpy() - exact_exp(A)).max() <= 2.0 ** -53 * 20 * d * (1 + 4 * norm), (norm, rep)
+            plan.close()
+    finally:
+        ctx.close()
+
+
+def test_batch_of_real_exponents_with_uneven_squarings():
+    rng = np.random.default_rng(3)
+    ctx = M.Context(0)
+    try:
+        As = [symmetric(rng, d, norm) for d, norm in ((40, 0.1), (45, 40.0), (48, 2.0), (70, 5.0), (33, 1e-3))]
+        plans, outs = [], []
+        for A in As:
+            p = M.Plan(ctx, torch.from_numpy(A).cuda(), None, M.MG_PREC_FP64)
+            p.set_controls(2, 1, 0.0, 0.5, np.array([2.0]), torch.zeros((2, 1, 0), dtype=torch.float64))
+            plans.append(p)
+            outs.append(torch.empty(A.shape, dtype=torch.complex128, device="cuda"))
+        assert M.mg_evolve_batch(ctx, plans, [M.MG_OUT_PROPAGATOR] * 5, [None] * 5, outs) == [0] * 5
+        torch.cuda.synchronize()
+        for A, o in zip(As, outs):
+            norm = np.abs(A - np.trace(A) / len(A) * np.eye(len(A))).sum(0).max()
+            assert np.abs(o.cpu().numpy() - exact_exp(A)).max() <= 2.0 ** -53 * 20 * 80 * (1 + 4 * norm)
     finally:
         ctx.close()
