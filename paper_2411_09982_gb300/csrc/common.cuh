@@ -131,11 +131,6 @@ int launch_cgemm_f64(int batch, int d, const double* A, long long strideA, int o
                      const double* B, long long strideB, double* C, long long strideC,
                      const AddTerms& add, cudaStream_t s);
 
-// the same for the items with mark_a[b] or mark_b[b] nonzero (device arrays) only
-int launch_cgemm_f64_marked(int batch, int d, const double* A, long long strideA, int opA, const double* B,
-                            long long strideB, double* C, long long strideC, const AddTerms& add, const int* mark_a,
-                            const int* mark_b, int sms, cudaStream_t s);
-
 // max-abs reductions used for reports: out = max_b max_ij |U_b^dag U_b - I| computed
 // from G_b = U_b^dag U_b (already formed), or |‖psi‖ - 1|.
 int launch_max_identity_defect(int batch, int d, const double* G, double* out_dev, cudaStream_t s);

@@ -25,18 +25,21 @@ struct AddDev {
   int sq_step;
 };
 
-// One TM x TM tile (origin i0, j0) of item b.
 template <int TM>
-__device__ __forceinline__ void cgemm_f64_tile(int b, int i0, int j0, int d, const double* __restrict__ A, long long sA,
-                                               int opA, const double* __restrict__ B, long long sB,
-                                               double* __restrict__ C, long long sC, const AddDev& add) {
+__global__ void __launch_bounds__(256)
+cgemm_f64_kernel(int d, const double* __restrict__ A, long long sA, int opA,
+                 const double* __restrict__ B, long long sB, double* __restrict__ C, long long sC,
+                 AddDev add) {
   constexpr int RT = TM / 16;                   // outputs per thread along each dimension
   constexpr int STAGE = (TM * FBK + 255) / 256; // staged elements per thread per operand
   __shared__ double2 As[FBK][TM];   // As[k][i] = opA(A)[i][k]
   __shared__ double2 Bs[FBK][TM];   // Bs[k][j] = B[k][j]
 
+  const int b = blockIdx.z;
+  if (add.item_sq && add.item_sq[b] <= add.sq_step) return;   // uniform over the CTA
   const double2* Ab = reinterpret_cast<const double2*>(A + b * sA);
   const double2* Bb = reinterpret_cast<const double2*>(B + b * sB);
+  const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TM;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
 
@@ -119,42 +122,11 @@ __device__ __forceinline__ void cgemm_f64_tile(int b, int i0, int j0, int d, con
   }
 }
 
-template <int TM>
-__global__ void __launch_bounds__(256)
-cgemm_f64_kernel(int d, const double* __restrict__ A, long long sA, int opA,
-                 const double* __restrict__ B, long long sB, double* __restrict__ C, long long sC,
-                 AddDev add) {
-  const int b = blockIdx.z;
-  if (add.item_sq && add.item_sq[b] <= add.sq_step) return;   // uniform over the CTA
-  cgemm_f64_tile<TM>(b, blockIdx.y * TM, blockIdx.x * TM, d, A, sA, opA, B, sB, C, sC, add);
-}
-
-// The items marked by the digit slicers (gemm_f64_digits.cu), usually none.  Every CTA looks
-// at all items, 256 at a time, and takes its share of the marked ones' tiles: a launch that
-// finds none costs 2-3 us whatever the batch (one CTA per tile and item took 13 us for 200
-// items of d = 256).
-__global__ void __launch_bounds__(256)
-cgemm_f64_marked_kernel(int batch, int d, const double* __restrict__ A, long long sA, int opA,
-                        const double* __restrict__ B, long long sB, double* __restrict__ C, long long sC,
-                        AddDev add, const int* __restrict__ mark_a, const int* __restrict__ mark_b) {
-  const int nt = (d + 63) / 64;
-  auto marked = [&](int b) {
-    return (mark_a[b] | mark_b[b]) != 0 && !(add.item_sq && add.item_sq[b] <= add.sq_step);
-  };
-  for (int b0 = 0; b0 < batch; b0 += 256) {
-    const int t = b0 + threadIdx.x;
-    if (!__syncthreads_or(t < batch && marked(t))) continue;
-    for (int b = b0; b < min(batch, b0 + 256); ++b) {
-      if (!marked(b)) continue;   // uniform over the CTA
-      // (item, tile) pairs in turn over the CTAs
-      const int before = (int)((long long)b * nt * nt % gridDim.x);
-      for (int tile = ((int)blockIdx.x - before + (int)gridDim.x) % (int)gridDim.x; tile < nt * nt; tile += gridDim.x)
-        cgemm_f64_tile<64>(b, (tile / nt) * 64, (tile % nt) * 64, d, A, sA, opA, B, sB, C, sC, add);
-    }
-  }
-}
-
-static AddDev add_dev(const AddTerms& add) {
+int launch_cgemm_f64(int batch, int d, const double* A, long long strideA, int opA, const double* B,
+                     long long strideB, double* C, long long strideC, const AddTerms& add,
+                     cudaStream_t s) {
+  if (batch <= 0) return MG_OK;
+  if (batch > 65535) return MG_EUNSUPPORTED;
   AddDev a{};
   a.n = add.n;
   for (int m = 0; m < 3; ++m) { a.src[m] = add.src[m]; a.coef[m] = add.coef[m]; }
@@ -163,24 +135,6 @@ static AddDev add_dev(const AddTerms& add) {
   a.scale = add.scale;
   a.item_sq = add.item_sq;
   a.sq_step = add.sq_step;
-  return a;
-}
-
-int launch_cgemm_f64_marked(int batch, int d, const double* A, long long strideA, int opA, const double* B,
-                            long long strideB, double* C, long long strideC, const AddTerms& add, const int* mark_a,
-                            const int* mark_b, int sms, cudaStream_t s) {
-  const long long tiles = (long long)ceil_div(d, 64) * ceil_div(d, 64) * batch;
-  cgemm_f64_marked_kernel<<<(int)(tiles < sms ? tiles : sms), 256, 0, s>>>(batch, d, A, strideA, opA, B, strideB, C,
-                                                                           strideC, add_dev(add), mark_a, mark_b);
-  return check_launch("cgemm_f64_marked_kernel");
-}
-
-int launch_cgemm_f64(int batch, int d, const double* A, long long strideA, int opA, const double* B,
-                     long long strideB, double* C, long long strideC, const AddTerms& add,
-                     cudaStream_t s) {
-  if (batch <= 0) return MG_OK;
-  if (batch > 65535) return MG_EUNSUPPORTED;
-  const AddDev a = add_dev(add);
   // tile edge: the smallest of 16, 32, 64 that covers d (64 beyond)
   if (d <= 16) {
     cgemm_f64_kernel<16><<<dim3(1, 1, batch), 256, 0, s>>>(d, A, strideA, opA, B, strideB, C, strideC, a);

@@ -20,19 +20,19 @@
 //     the slicers record per item.  Full random digits give n = 12 and 18 (levels 0..3),
 //     whatever the operands 6 and 10 steps are exact, and most matrices of the exponential
 //     take one drain per sweep.
-//   * The two 64-bit sums (levels 0..3 and 4..7) are joined by one FP64 FMA, the product's
-//     only rounding beside that of F.
+//   * The two 64-bit sums (levels 0..3 and 4..7) are joined and rounded to FP64 on the integer
+//     pipe, the product's only rounding beside that of F.
 // The error is about 2^-58 of (largest entry of the row of A) x (largest entry of the column
 // of B) beside the rounding of the result: below FP64 arithmetic's, whose K roundings
 // accumulate.  Whole evolutions against quad precision (relative 2-norm, here / FP64 pipe):
 // spin chain d = 64, six squarings per interval 2.1e-14 / 5.6e-14, four 4.4e-15 / 3.2e-14;
 // transmon chain d = 81 2.7e-14 / 1.1e-13; transmon-resonator d = 80 1.1e-12 / 1.6e-12.
 // (Base-128 digits, 56 bits, need fewer drains but gave 2.3e-14, 1.3e-14, 1.0e-13, 1.1e-12.)
-// Operands that the scheme does not cover -- a NaN, an infinity, a row or column whose largest entry lies outside 2^-400 .. 2^400 -- are marked
-// by the slicers; such an item is left to the FP64-pipe product, which is launched behind
-// and returns at once for all others.
+// Operands that the scheme does not cover -- a NaN, an infinity, a row or column whose largest
+// entry lies outside 2^-400 .. 2^400 -- are marked by the slicers; the epilogue warps compute
+// such an item in FP64 arithmetic (f8_pipe_row).
 //
-// Structure of the product kernel (persistent, one CTA of 320 threads per SM, 128 x 64
+// Structure of the product kernel (persistent, one CTA of 640 threads per SM, 128 x 64
 // complex output tiles; every tile makes two sweeps over K, levels 4..7 first):
 //   warp 0      TMA producer: 32 KiB slots (4 digits of the A or B tile, K = 32, SWIZZLE_64B)
 //               in a ring of six.  Levels 0..3 need the digits 0..3 of A and B (two slots per
@@ -42,17 +42,17 @@
 //               (A 0..3, B 0..3), (A 0..3, B 4..7), (A 4..7, B 0..3) frees two slots while
 //               ten digit pairs are still to be multiplied, so a ring of 1.5 K steps keeps
 //               loads in flight.
-//   warps 2..9  drains: tcgen05.ld, float -> int, 64-bit accumulation in registers (64 sums
-//               per thread).  The sums of levels 4..7 wait in a per-CTA scratch (L2) while
-//               levels 0..3 are swept.  Conversion to FP64, scaling, addends and stores run
-//               while the next tile's MMAs are issued: the FP64 pipe (4 operations per output)
-//               is idle otherwise.
+//   warps 4..19 drains: tcgen05.ld, float -> int, 64-bit accumulation in registers (32 sums
+//               per thread).  The low words of levels 4..7 wait in a per-CTA scratch (L2)
+//               while levels 0..3 are swept onto the high ones.  Rounding to FP64, addends
+//               and stores run while the next tile's MMAs are issued.  These warps take
+//               registers over from the first four (setmaxnreg).
 // Measured (GB300, one product of a batch, slicing included): d = 729 2804 us on the FP64
-// pipe -> 109 us (28 TFLOP/s of the product's 8 d^3); d = 256 112 -> 8.8 us; d = 81 8.9 ->
-// 1.5 us.  At d = 729 the slicers take 12% (HBM-bound) and the tensor pipe is active about
-// two thirds of the product's cycles: the rest goes to the drains (~5000 cycles each,
-// float-to-int conversions above all) and to operand delivery (single CTAs load 43 bytes per
-// cycle and SM).
+// pipe -> 106 us (29 TFLOP/s of the product's 8 d^3); d = 256 112 -> 7.6 us; d = 81 8.9 ->
+// 1.2 us.  Small K is bound by the epilogue's latency, which is why it has 16 warps (eight
+// warps of 64 sums: d = 84 exponentials 2.93 -> 2.42 ms, d = 256 12.1 -> 10.7, d = 729 the
+// same); at d = 729 the slicers take 12% (HBM-bound), the drains 11%, and the operands arrive
+// at 43 bytes per cycle and SM, near what L2 delivers.
 // Every wait is bounded (SplitCtl::wait_ns, at most 4 s): a wait that gives up records
 // MG_DEV_TIMEOUT, the CTA's unfinished tiles become NaN, and it leaves once its own copies
 // and MMAs have completed.
@@ -71,12 +71,18 @@ constexpr int F8_BN = 64;               // complex output columns per tile
 constexpr int F8_BK = 32;               // K per slot
 constexpr int F8_SLOTS = 6;
 constexpr int F8_SLOT_BYTES = 4 * F8_BM * F8_BK * 2;
-constexpr int F8_THREADS = 320;
-constexpr int F8_EPI_WARPS = 8;
+constexpr int F8_THREADS = 640;         // warps 0..3: loads, MMAs (two idle); warps 4..19: drains and epilogue
+constexpr int F8_EPI_WARPS = 16;
 constexpr int F8_SEG_LO = 6;            // K steps per drain of levels 4..7 that are exact whatever the digits
 constexpr int F8_SEG_HI = 10;           // and of levels 0..3
-constexpr int F8_VALS = 64;             // sums per epilogue thread
-constexpr int F8_STAGE_BYTES = F8_EPI_WARPS * 32 * 8 * 16;   // epilogue staging: 32 rows x 8 columns per warp
+constexpr int F8_VALS = 32;             // sums per epilogue thread
+constexpr int F8_EPI = F8_EPI_WARPS * 32;
+constexpr int F8_STAGE_BYTES = F8_EPI_WARPS * 2048;   // epilogue staging: 32 rows x 4 complex (8 real) columns per warp
+// Register split (setmaxnreg): the launch holds 640 x 96 = 128 x 64 + 512 x 104
+constexpr int F8_REGS_LAUNCH = 96;
+constexpr int F8_REGS_IO = 64;
+constexpr int F8_REGS_EPI = 104;
+static_assert(128 * F8_REGS_IO + F8_EPI * F8_REGS_EPI <= F8_THREADS * F8_REGS_LAUNCH, "a larger split would wait forever");
 constexpr int F8_EXP_MAX = 400;
 
 struct F8Geom {
@@ -91,6 +97,17 @@ static F8Geom f8_geom(int d) {
   g.a_elems = (long long)F8_L * d * g.Kp;        // rows [Re | 0 | Im | 0]
   g.b_elems = (long long)F8_L * 3 * d * g.Kh;    // planes -Im, Re, Im of the columns
   return g;
+}
+
+// The product's kernels have to be compiled to the register count their split starts from.
+static int f8_check_registers(const void* kern) {
+  cudaFuncAttributes at;
+  MG_CUDA_TRY(cudaFuncGetAttributes(&at, kern));
+  if (at.numRegs < F8_REGS_LAUNCH) {
+    set_last_message("the FP64 digit product is compiled to %d registers, its split needs %d", at.numRegs, F8_REGS_LAUNCH);
+    return MG_EUNSUPPORTED;
+  }
+  return MG_OK;
 }
 
 // operand buffer: digits of all items, then row (column) exponents, then the items' marks and
@@ -110,6 +127,9 @@ __device__ __forceinline__ int f8_exp(double a) {
   const int bexp = (__double2hiint(a) >> 20) & 0x7FF;
   return bexp == 0 ? -(1 << 29) : bexp - 1022;
 }
+// exponents are stored as E + 4096; 0 is a row or column without a nonzero entry
+constexpr int F8_EBIAS = 4096;
+__device__ __forceinline__ int f8_exponent(int stored) { return stored ? stored - F8_EBIAS : 0; }
 __device__ __forceinline__ bool f8_marked(int E) { return E > F8_EXP_MAX || (E < -F8_EXP_MAX && E > -(1 << 28)); }
 
 constexpr unsigned long long F8_BIAS = 0x8080808080808080ull;   // 128 in every base-256 position
@@ -196,7 +216,7 @@ f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2,
   const bool mark = f8_marked(E);
   if (E < -(1 << 28)) E = 0;   // all-zero row
   if (lane == 0) {
-    ea[(long long)b * d + row] = E;
+    ea[(long long)b * d + row] = E + F8_EBIAS;
     if (mark) atomicOr(bad + b, 1);
   }
   __nv_bfloat16* o = out + b * item_elems + (long long)row * Kp;
@@ -224,7 +244,7 @@ f64d_slice_a_kernel(int d, int Kp, const double2* __restrict__ A, long long sA2,
   f8_energy_store(en, energy + 2 * b, lane);
 }
 
-// Column exponents (preset to byte 0x80): grid (ceil(d/64), ceil(d/64), batch), block 256.
+// Column exponents (preset to 0): grid (ceil(d/64), ceil(d/64), batch), block 256.
 __global__ void __launch_bounds__(256)
 f64d_col_exponent_kernel(int d, const double2* __restrict__ B, long long sB2, int* __restrict__ eb,
                          const int* __restrict__ item_sq, int sq_step) {
@@ -241,8 +261,10 @@ f64d_col_exponent_kernel(int d, const double2* __restrict__ B, long long sB2, in
     }
   red[g][c] = E;
   __syncthreads();
-  if (g == 0 && j0 + c < d)
-    atomicMax(eb + (long long)b * d + j0 + c, max(max(red[0][c], red[1][c]), max(red[2][c], red[3][c])));
+  if (g == 0 && j0 + c < d) {
+    E = max(max(red[0][c], red[1][c]), max(red[2][c], red[3][c]));
+    if (E > -(1 << 28)) atomicMax(eb + (long long)b * d + j0 + c, E + F8_EBIAS);
+  }
 }
 
 // Column digits of a 32 (k) x 64 (j) block, staged in shared memory.  ADJ = false: B planes
@@ -260,9 +282,9 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
   const int j0 = blockIdx.x * 64, k0 = blockIdx.y * 32, tid = threadIdx.x, Kh = Kp / 2;
   const double2* Bb = B + b * sB2;
   if (tid < 64) {
-    int E = j0 + tid < d ? eb[(long long)b * d + j0 + tid] : 0;
+    const int E = j0 + tid < d ? f8_exponent(eb[(long long)b * d + j0 + tid]) : 0;
     if (f8_marked(E)) atomicOr(bad + b, 1);
-    ex[tid] = E < -(1 << 28) ? 0 : E;   // all-zero column
+    ex[tid] = E;
   }
   for (int e = tid; e < 32 * 64; e += 256) {
     const int kk = e >> 6, c = e & 63;
@@ -308,7 +330,6 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
     }
   }
   f8_energy_store(en, energy + 2 * b, tid & 31);
-  // the exponents of all-zero columns stay preset; the product reads them as 0
 }
 
 // Row digits of a real symmetric matrix (both operands of its products are such rows), one
@@ -336,7 +357,7 @@ f64r_slice_kernel(int d, int Kh, const double* __restrict__ X, const double* __r
   const int s = CW ? (sq_dev ? sq_dev[b] : sq) : 0;
   if (E < -(1 << 28)) E = s;                 // all-zero row
   E = max(E, s - F8_EXP_MAX);
-  if (lane == 0) ex[(long long)b * d + row] = E - s;
+  if (lane == 0) ex[(long long)b * d + row] = E - s + F8_EBIAS;
   __nv_bfloat16* o = out + b * item_elems + (long long)row * Kh;
   const long long ds = (long long)d * Kh;
   uint32_t en = 0;
@@ -404,6 +425,10 @@ f64r_phase_kernel(long long per, const double* __restrict__ tau, const double* _
 // product
 // ---------------------------------------------------------------------------
 struct F8Args {
+  const double* A;            // the operands themselves, for marked items (complex products)
+  const double* B;
+  long long sA, sB;           // doubles
+  int opA;
   int d, Kp, batch, ntn, ntm;   // Kp: length of the K axis; per item ntm x ntn tiles
   const int* ea;
   const int* eb;
@@ -417,8 +442,9 @@ struct F8Args {
   double add_coef[3];
   long long add_stride;       // doubles
   int add_n;
-  double diag, scale;         // scale: real products only
-  long long* scratch;         // per CTA: F8_VALS x 256 sums of levels 4..7
+  double diag;
+  int scale2;                 // real products only: the product times 2^scale2
+  uint32_t* scratch;          // per CTA: the low words of F8_VALS x F8_EPI sums of levels 4..7
   int* status;
   const int* item_sq;
   int sq_step;
@@ -428,6 +454,34 @@ struct F8Args {
 
 __device__ __forceinline__ bool f8_skip(const F8Args& p, int b) {
   return (p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.item_sq && p.item_sq[b] <= p.sq_step);
+}
+
+// One row's columns c0 .. c1 of a marked item in FP64 arithmetic, in the order of
+// cgemm_f64_kernel (the same bits).
+__device__ __noinline__ void f8_pipe_row(const F8Args& p, int b, int row, int c0, int c1) {
+  const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
+  const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
+  double2* C = reinterpret_cast<double2*>(p.C + b * p.sC);
+  for (int c = c0; c < c1; ++c) {
+    double re = 0.0, im = 0.0;
+    for (int k = 0; k < p.d; ++k) {
+      double2 x = p.opA ? A[(long long)k * p.d + row] : A[(long long)row * p.d + k];
+      if (p.opA) x.y = -x.y;
+      const double2 y = B[(long long)k * p.d + c];
+      re = fma(x.x, y.x, re);
+      re = fma(-x.y, y.y, re);
+      im = fma(x.x, y.y, im);
+      im = fma(x.y, y.x, im);
+    }
+    const long long off = (long long)row * p.d + c;
+    for (int m = 0; m < p.add_n; ++m) {
+      const double2 v = reinterpret_cast<const double2*>(p.add_src[m] + b * p.add_stride)[off];
+      re = fma(p.add_coef[m], v.x, re);
+      im = fma(p.add_coef[m], v.y, im);
+    }
+    if (row == c) re += p.diag;
+    C[off] = make_double2(re, im);
+  }
 }
 
 // polls until the phase completes, the CTA aborts or the limit runs out
@@ -440,9 +494,37 @@ __device__ __forceinline__ bool f8_wait(uint64_t* bar, uint32_t parity, unsigned
   return true;
 }
 
-// 64-bit integer |x| < 2^51 as FP64 (exact): the bits of 1.5 2^52 + x
-__device__ __forceinline__ double f8_to_double(long long x) {
-  return __longlong_as_double(x + 0x4338000000000000ll) - 6755399441055744.0;
+// (t 2^32 + w) 2^k rounded to FP64, |t| < 2^63; k keeps the result a normal number.
+__device__ __forceinline__ double f8_value(long long t, uint32_t w, int k) {
+  const uint32_t neg = (uint32_t)((unsigned long long)t >> 63);
+  const unsigned long long s = 0ull - neg;
+  w = (w ^ (uint32_t)s) + neg;                                   // |T|, 96 bits
+  unsigned long long u = ((unsigned long long)t ^ s) + (neg & (w == 0u));
+  uint32_t t1 = (uint32_t)(u >> 32), t0 = (uint32_t)u;
+  int e = k + 95 + 1022;                                         // biased exponent less one if t1's top bit is set
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const bool z = t1 == 0u;
+    t1 = z ? t0 : t1;
+    t0 = z ? w : t0;
+    w = z ? 0u : w;
+    e -= z ? 32 : 0;
+  }
+  const int lz = __clz((int)t1);
+  const uint32_t m1 = __funnelshift_l(t0, t1, lz), m0 = __funnelshift_l(w, t0, lz);   // 64 bits, the top one set
+  // 53 bits and the rounding bit; a carry runs into the exponent as it should
+  const unsigned long long m = ((unsigned long long)m1 << 32 | m0) >> 11;
+  const unsigned long long bits = ((unsigned long long)(uint32_t)(e - lz) << 52) + m + ((m0 >> 10) & 1u);
+  return t1 == 0u ? 0.0 : __longlong_as_double((long long)(bits | (unsigned long long)neg << 63));
+}
+
+// The same on the FP64 pipe, |t| < 2^51.  A warp's FP64 instruction takes about 68 cycles of
+// its quarter of the SM, the integer form some 50 dependent instructions: the epilogues send
+// every fourth value here, which is where the two balance.
+__device__ __forceinline__ double f8_value_fp64(long long t, uint32_t w, int k) {
+  const double h = __longlong_as_double(t + 0x4338000000000000ll) - 6755399441055744.0;   // (1.5 2^52 + t) - 1.5 2^52
+  const double l = __hiloint2double(0x43300000, (int)w) - 4503599627370496.0;             // (2^52 + w) - 2^52
+  return fma(h, 4294967296.0, l) * __hiloint2double((k + 1023) << 20, 0);
 }
 
 // Drain of one accumulator set (levels l0 .. l0 + 3) into the thread's sums, in units of
@@ -452,16 +534,16 @@ __device__ __forceinline__ void f8_drain(uint32_t tbase, int l0, long long (&acc
   const float m0 = l0 ? 4294967296.0f : 1.0f;   // 2^{8 l0}
   const float m1 = m0 * 256.0f, m2 = m0 * 65536.0f, m3 = m0 * 16777216.0f;
 #pragma unroll
-  for (int c = 0; c < F8_VALS; c += 8) {
-    // complex: values 0..31 are the real parts of the thread's 32 columns, 32..63 the imaginary
-    // parts; real: 64 columns
-    const uint32_t col = tbase + (CPLX && c >= 32 ? F8_BN + c - 32 : c);
-    uint32_t g[4][8];
+  for (int c = 0; c < F8_VALS; c += 4) {
+    // complex: values 0..15 are the real parts of the thread's 16 columns, 16..31 the imaginary
+    // parts; real: 32 columns
+    const uint32_t col = tbase + (CPLX && c >= F8_VALS / 2 ? F8_BN + c - F8_VALS / 2 : c);
+    uint32_t g[4][4];
 #pragma unroll
-    for (int l = 0; l < 4; ++l) tmem_ld8(col + l * 128, g[l]);
+    for (int l = 0; l < 4; ++l) tmem_ld4(col + l * 128, g[l]);
     tmem_wait_ld();
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
+    for (int v = 0; v < 4; ++v) {
       acc[c + v] += (long long)__float2int_rn(__uint_as_float(g[0][v]) * m0) * 16777216 +
                     (long long)__float2int_rn(__uint_as_float(g[1][v]) * m1) * 65536;
       acc[c + v] += (long long)__float2int_rn(__uint_as_float(g[2][v]) * m2) * 256 +
@@ -536,6 +618,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     return (steps + n - 1) / n;
   };
 
+  if (warp < 4) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F8_REGS_IO));
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer ----------------
@@ -662,15 +746,17 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       while (!mbar_try_wait(mmadone, 0) && global_ns() - t0 < 4000000000ull) {
       }
     }
+  }
   } else {
-    // ---------------- epilogue (warps 2..9) ----------------
+    // ---------------- epilogue (warps 4..19) ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F8_REGS_EPI));
     const int q = warp & 3;                    // TMEM lane quarter of this warp
-    constexpr int WC = CPLX ? 32 : 64;         // columns per warp
-    const int c0 = ((warp - 2) >> 2) * WC;
-    const int et = threadIdx.x - 64;
+    constexpr int WC = CPLX ? 16 : 32;         // columns per warp, four warps to a tile's row
+    const int c0 = ((warp - 4) >> 2) * WC;
+    const int et = threadIdx.x - 128;
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + c0;
-    long long* scratch = p.scratch + (long long)blockIdx.x * F8_VALS * 256 + et;
-    double2* stg = staging + (warp - 2) * 256;
+    uint32_t* scratch = p.scratch + (long long)blockIdx.x * F8_VALS * F8_EPI + et;
+    double2* stg = staging + (warp - 4) * 128;
     uint32_t set = 0;
     bool ok = true;
     long long t = blockIdx.x;
@@ -678,14 +764,19 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int b = (int)(t / per_item);
       int mt, nt;
       f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
-      if (f8_skip(p, b)) continue;
-      const int row0 = mt * F8_BM + q * 32, col0 = nt * 2 * WC + c0;
+      const int row0 = mt * F8_BM + q * 32, col0 = nt * 4 * WC + c0;
+      if (f8_skip(p, b)) {
+        if constexpr (CPLX)
+          if ((p.bad_a[b] | p.bad_b[b]) != 0 && !(p.item_sq && p.item_sq[b] <= p.sq_step) && row0 + lane < p.d)
+            f8_pipe_row(p, b, row0 + lane, col0, min(p.d, col0 + WC));
+        continue;
+      }
       // uniform over the warp; a real tile's columns right of all its rows are not needed
       const bool live = row0 < p.d && col0 < p.d && (CPLX || col0 <= row0 + 31);
       long long acc[F8_VALS];
-      for (int sweep = 0; sweep < 2 && ok; ++sweep) {
 #pragma unroll
-        for (int v = 0; v < F8_VALS; ++v) acc[v] = 0;
+      for (int v = 0; v < F8_VALS; ++v) acc[v] = 0;
+      for (int sweep = 0; sweep < 2 && ok; ++sweep) {
         const int ns = segments(b, sweep);
         for (int sg = 0; sg < ns; ++sg) {
           bool got = true;
@@ -701,39 +792,58 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           ++set;
         }
         if (sweep == 0 && ok && live) {
+          // the levels 4..7, in units of 2^-56: the sums of levels 0..3, in units of 2^-24, go
+          // on from their high words; the low words wait in the scratch
 #pragma unroll
-          for (int v = 0; v < F8_VALS; ++v) scratch[v * 256] = acc[v];
+          for (int v = 0; v < F8_VALS; ++v) {
+            scratch[v * F8_EPI] = (uint32_t)acc[v];
+            acc[v] >>= 32;
+          }
+          if (p.add_n > 0) {   // the tile's addends into L2 (128-byte lines)
+            const int lines = 2, n = p.add_n * 32 * lines;
+            const int r0 = CPLX ? row0 : col0, q0 = CPLX ? col0 : row0;   // real addends are read as columns
+            for (int i = lane; i < n; i += 32) {
+              const int m = i / (32 * lines), r = r0 + i / lines % 32, c = q0 + (i % lines) * (CPLX ? 8 : 16);
+              if (r < p.d && c < p.d)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"((m == 0 ? p.add_src[0] : m == 1 ? p.add_src[1] : p.add_src[2]) +
+                                                              b * p.add_stride + ((long long)r * p.d + c) * (CPLX ? 2 : 1)));
+            }
+          }
         }
       }
       if (!ok) break;
       if (!live) continue;
       const int row = row0 + lane;
-      const int Ea = row < p.d ? p.ea[(long long)b * p.d + row] : 0;
+      const int Ea = row < p.d ? f8_exponent(p.ea[(long long)b * p.d + row]) : 0;
       if constexpr (!CPLX) {
         // entry (row, col) goes to both sides of the diagonal: (col, row) straight from the
         // registers (lanes are consecutive rows), (row, col) through the warp's staging
         double* Cr = p.C + b * p.sC;
         double* stg8 = reinterpret_cast<double*>(stg);
         const int* ebp = p.eb + (long long)b * p.d;
+        uint32_t lo[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) lo[v] = scratch[v * F8_EPI];
 #pragma unroll
         for (int c = 0; c < F8_VALS; c += 8) {
-          if (col0 + c < p.d && col0 + c <= row0 + 31) {
-            long long lo[8];
+          uint32_t w[8];
 #pragma unroll
-            for (int v = 0; v < 8; ++v) lo[v] = scratch[(c + v) * 256];
+          for (int v = 0; v < 8; ++v) {
+            w[v] = lo[v];
+            if (c + 8 < F8_VALS) lo[v] = scratch[(c + 8 + v) * F8_EPI];   // one round ahead
+          }
+          if (col0 + c < p.d && col0 + c <= row0 + 31) {
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
               const int col = col0 + c + v;
-              const int k = Ea + (col < p.d ? ebp[col] : 0) - 64;
-              double x = fma(f8_to_double(acc[c + v]), 268435456.0, f8_to_double(lo[v] >> 4)) *
-                         __hiloint2double((k + 1023) << 20, 0);
+              const int k = Ea + (col < p.d ? f8_exponent(ebp[col]) : 0) - 68 + p.scale2;
+              double x = v % 4 == 3 ? f8_value_fp64(acc[c + v], w[v], k) : f8_value(acc[c + v], w[v], k);
               if (row < p.d && col <= row) {
                 const long long off = (long long)col * p.d + row;
 #pragma unroll
                 for (int m = 0; m < 3; ++m)
                   if (m < p.add_n) x = fma(p.add_coef[m], p.add_src[m][b * p.add_stride + off], x);
                 if (col == row) x += p.diag;
-                x *= p.scale;
                 Cr[off] = x;
               }
               stg8[lane * 8 + (v ^ (lane & 7))] = x;
@@ -749,38 +859,47 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
         }
       } else {
-      int Eb = col0 + lane < p.d ? p.eb[(long long)b * p.d + col0 + lane] : 0;
-      if (Eb < -(1 << 28)) Eb = 0;   // all-zero column
+      const int Eb = col0 + lane < p.d ? f8_exponent(p.eb[(long long)b * p.d + col0 + lane]) : 0;
       const double2* addp[3];
 #pragma unroll
       for (int m = 0; m < 3; ++m)
         addp[m] = reinterpret_cast<const double2*>(m < p.add_n ? p.add_src[m] + b * p.add_stride : nullptr);
       double2* Cb = reinterpret_cast<double2*>(p.C + b * p.sC);
+      uint32_t lre[4], lim[4];
 #pragma unroll
-      for (int c = 0; c < 32; c += 8) {   // 8 columns at a time through the warp's staging
-        if (col0 + c < p.d) {
-          long long lre[8], lim[8];
+      for (int v = 0; v < 4; ++v) {
+        lre[v] = scratch[v * F8_EPI];
+        lim[v] = scratch[(WC + v) * F8_EPI];
+      }
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            lre[v] = scratch[(c + v) * 256];
-            lim[v] = scratch[(32 + c + v) * 256];
+      for (int c = 0; c < WC; c += 4) {   // 4 columns at a time through the warp's staging
+        uint32_t wre[4], wim[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          wre[v] = lre[v];
+          wim[v] = lim[v];
+          if (c + 4 < WC) {   // one round ahead
+            lre[v] = scratch[(c + 4 + v) * F8_EPI];
+            lim[v] = scratch[(WC + 4 + c + v) * F8_EPI];
           }
+        }
+        if (col0 + c < p.d) {
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            // the value is T 2^{Ea + Eb - 64}, T = hi 2^28 + lo / 2^4 in units of 2^-52
-            const int k = Ea + __shfl_sync(0xffffffffu, Eb, c + v) - 64;
-            const double sc = __hiloint2double((k + 1023) << 20, 0);
-            const double re = fma(f8_to_double(acc[c + v]), 268435456.0, f8_to_double(lre[v] >> 4)) * sc;
-            const double im = fma(f8_to_double(acc[32 + c + v]), 268435456.0, f8_to_double(lim[v] >> 4)) * sc;
-            stg[lane * 8 + (v ^ (lane & 7))] = make_double2(re, im);
+          for (int v = 0; v < 4; ++v) {
+            // the value is (sum 2^32 + low word) 2^{Ea + Eb - 68}, in units of 2^-56; every
+            // fourth goes over the FP64 pipe
+            const int k = Ea + __shfl_sync(0xffffffffu, Eb, c + v) - 68;
+            const double re = f8_value(acc[c + v], wre[v], k);
+            const double im = v & 1 ? f8_value_fp64(acc[WC + c + v], wim[v], k) : f8_value(acc[WC + c + v], wim[v], k);
+            stg[lane * 4 + (v ^ ((lane >> 1) & 3))] = make_double2(re, im);
           }
           __syncwarp();
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = i * 4 + (lane >> 3), cc = lane & 7;
+          for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + (lane >> 2), cc = lane & 3;
             const int grow = row0 + r, gcol = col0 + c + cc;
             if (grow < p.d && gcol < p.d) {
-              double2 v = stg[r * 8 + (cc ^ (r & 7))];
+              double2 v = stg[r * 4 + (cc ^ ((r >> 1) & 3))];
               const long long off = (long long)grow * p.d + gcol;
 #pragma unroll
               for (int m = 0; m < 3; ++m)
@@ -811,7 +930,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         const int row = mt * F8_BM + q * 32 + lane;
         if (f8_skip(p, b) || row >= p.d) continue;
-        const int n0 = nt * 2 * WC + c0;
+        const int n0 = nt * 4 * WC + c0;
         for (int c = n0; c < min(p.d, n0 + WC); ++c) {
           if constexpr (CPLX) reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
           else p.C[b * p.sC + (long long)row * p.d + c] = p.C[b * p.sC + (long long)c * p.d + row] = nan;
@@ -859,8 +978,7 @@ int f64d_slice_a(int d, int batch, const double* A, long long sA, int opA, void*
                                                                     o.energy, ctl.item_sq, ctl.sq_step);
     return check_launch("f64d_slice_a_kernel");
   }
-  MG_CUDA_TRY(cudaMemsetAsync(o.e, 0x80, sizeof(int) * (size_t)d * batch, s));
-  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, 3 * sizeof(int) * (size_t)batch, s));
+  MG_CUDA_TRY(cudaMemsetAsync(o.e, 0, sizeof(int) * (size_t)(d + 3) * batch, s));   // exponents, marks, energies
   f64d_col_exponent_kernel<<<dim3(ceil_div(d, 64), ceil_div(d, 64), batch), 256, 0, s>>>(d, A2, sA / 2, o.e,
                                                                                           ctl.item_sq, ctl.sq_step);
   MG_TRY(check_launch("f64d_col_exponent_kernel"));
@@ -874,8 +992,7 @@ int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cud
   const F8Geom g = f8_geom(d);
   const F8Buf o = f8_buf(buf, g.b_elems, d, batch);
   const double2* B2 = reinterpret_cast<const double2*>(B);
-  MG_CUDA_TRY(cudaMemsetAsync(o.e, 0x80, sizeof(int) * (size_t)d * batch, s));
-  MG_CUDA_TRY(cudaMemsetAsync(o.bad, 0, 3 * sizeof(int) * (size_t)batch, s));
+  MG_CUDA_TRY(cudaMemsetAsync(o.e, 0, sizeof(int) * (size_t)(d + 3) * batch, s));   // exponents, marks, energies
   f64d_col_exponent_kernel<<<dim3(ceil_div(d, 64), ceil_div(d, 64), batch), 256, 0, s>>>(d, B2, sB / 2, o.e,
                                                                                           ctl.item_sq, ctl.sq_step);
   MG_TRY(check_launch("f64d_col_exponent_kernel"));
@@ -884,8 +1001,8 @@ int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cud
   return check_launch("f64d_slice_col_kernel");
 }
 
-// scratch of the product (sums of levels 4..7 between the sweeps): one block per SM
-size_t f64d_scratch_bytes(int sms) { return (size_t)sms * F8_VALS * 256 * sizeof(long long); }
+// scratch of the product (low words between the sweeps): one block per SM
+size_t f64d_scratch_bytes(int sms) { return (size_t)sms * F8_VALS * F8_EPI * sizeof(uint32_t); }
 
 int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const void* abuf, const double* B,
               long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
@@ -900,6 +1017,11 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   MG_TRY(make_digit_map(&ma, a.dig, g.Kp, d, d, F8_L, batch, F8_BK, F8_BM, 4));
   MG_TRY(make_bplane_map(&mb, b.dig, g.Kh, d, d, F8_L, batch, 2, 4, F8_BK));
   F8Args p{};
+  p.A = A;
+  p.B = B;
+  p.sA = sA;
+  p.sB = sB;
+  p.opA = opA;
   p.d = d;
   p.Kp = g.Kp;
   p.batch = batch;
@@ -917,7 +1039,7 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   for (int m = 0; m < 3; ++m) { p.add_src[m] = add.src[m]; p.add_coef[m] = add.coef[m]; }
   p.add_stride = add.stride;
   p.diag = add.diag;
-  p.scratch = reinterpret_cast<long long*>(scratch);
+  p.scratch = reinterpret_cast<uint32_t*>(scratch);
   p.status = status;
   p.item_sq = ctl.item_sq;
   p.sq_step = ctl.sq_step;
@@ -927,13 +1049,10 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   const int grid = (int)std::min<long long>(tiles, sms);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<true>), (int)smem));
+  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<true>)));
   f64d_gemm_kernel<true><<<grid, F8_THREADS, smem, s>>>(ma, mb, p);
   MG_TRY(check_launch("f64d_gemm_kernel"));
-  // items the slicers marked (usually none: the launch returns at once)
-  AddTerms rest = add;
-  rest.item_sq = ctl.item_sq;
-  rest.sq_step = ctl.sq_step;
-  return launch_cgemm_f64_marked(batch, d, A, sA, opA, B, sB, C, sC, rest, a.bad, b.bad, sms, s);
+  return MG_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -982,9 +1101,10 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
   const int ntm = ceil_div(d, F8_BM);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<false>), (int)smem));
-  // dst = scale (D[x] D[y] + sum_m coef_m src_m + diag I)
+  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<false>)));
+  // dst = 2^scale2 D[x] D[y] + sum_m coef_m src_m + diag I
   auto mul = [&](int x, int y, double* dst, int n, const double* const* src, const double* coef, double diag,
-                 double scale) {
+                 int scale2) {
     F8Args p{};
     p.d = d;
     p.Kp = Kh;
@@ -1000,8 +1120,8 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
     for (int q = 0; q < n; ++q) { p.add_src[q] = src[q]; p.add_coef[q] = coef[q]; }
     p.add_stride = dd;
     p.diag = diag;
-    p.scale = scale;
-    p.scratch = reinterpret_cast<long long*>(scratch);
+    p.scale2 = scale2;
+    p.scratch = reinterpret_cast<uint32_t*>(scratch);
     p.status = status;
     p.item_sq = ctl.item_sq;
     p.sq_step = ctl.sq_step;
@@ -1026,16 +1146,16 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
   f64r_slice_kernel<true><<<dim3(ceil_div(d, 8), batch), 256, 0, s>>>(d, Kh, W, nullptr, 0.0, 2 * dd, sq, sq_dev, D[0].dig,
                                                                       elems, D[0].e, D[0].energy, nullptr, 0);
   MG_TRY(check_launch("f64r_slice_kernel"));
-  MG_TRY(mul(0, 0, Y[0], 0, nullptr, nullptr, 0.0, 1.0));
+  MG_TRY(mul(0, 0, Y[0], 0, nullptr, nullptr, 0.0, 0));
   int dp = 1;   // digits of Y^p
   if (p >= 2 || hc || hs) MG_TRY(slice(1, Y[0], nullptr, 0.0));
   if (p >= 2) {
-    MG_TRY(mul(1, 1, Y[1], 0, nullptr, nullptr, 0.0, 1.0));
+    MG_TRY(mul(1, 1, Y[1], 0, nullptr, nullptr, 0.0, 0));
     MG_TRY(slice(2, Y[1], nullptr, 0.0));
     dp = 2;
   }
-  if (p >= 3) MG_TRY(mul(2, 1, Y[2], 0, nullptr, nullptr, 0.0, 1.0));
-  if (p >= 4) MG_TRY(mul(2, 2, Y[3], 0, nullptr, nullptr, 0.0, 1.0));
+  if (p >= 3) MG_TRY(mul(2, 1, Y[2], 0, nullptr, nullptr, 0.0, 0));
+  if (p >= 4) MG_TRY(mul(2, 2, Y[3], 0, nullptr, nullptr, 0.0, 0));
   if (p >= 3) MG_TRY(slice(2, Y[p - 1], nullptr, 0.0));
   RealComb a{};
   a.n = p;
@@ -1055,16 +1175,16 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
   const int hd = dp == 1 ? 3 : 1;   // where the high part's digits go
   if (hc) {
     MG_TRY(slice(hd, T1, nullptr, 0.0));
-    MG_TRY(mul(hd, dp, C, p - 1, low, cc + 1, cc[0], 1.0));
+    MG_TRY(mul(hd, dp, C, p - 1, low, cc + 1, cc[0], 0));
   }
   double* sine = T2;
   if (hs) {
     MG_TRY(slice(hd, T2, nullptr, 0.0));
-    MG_TRY(mul(hd, dp, S, p - 1, low, ss + 1, ss[0], 1.0));
+    MG_TRY(mul(hd, dp, S, p - 1, low, ss + 1, ss[0], 0));
     sine = S;
   }
   MG_TRY(slice(3, sine, nullptr, 0.0));
-  MG_TRY(mul(0, 3, S, 0, nullptr, nullptr, 0.0, 1.0));   // sin = A (sum)
+  MG_TRY(mul(0, 3, S, 0, nullptr, nullptr, 0.0, 0));   // sin = A (sum)
   for (int k = 0; k < sq; ++k) {
     ctl.item_sq = sq_dev;   // items whose count is reached keep their matrices
     ctl.sq_step = k;
@@ -1072,8 +1192,8 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
     MG_TRY(slice(1, C, S, -1.0));
     MG_TRY(slice(2, S, nullptr, 0.0));
     MG_TRY(slice(3, C, nullptr, 0.0));
-    MG_TRY(mul(0, 1, C, 0, nullptr, nullptr, 0.0, 1.0));
-    MG_TRY(mul(2, 3, S, 0, nullptr, nullptr, 0.0, 2.0));
+    MG_TRY(mul(0, 1, C, 0, nullptr, nullptr, 0.0, 0));
+    MG_TRY(mul(2, 3, S, 0, nullptr, nullptr, 0.0, 1));
   }
   f64r_phase_kernel<<<dim3((unsigned)std::min<long long>((dd + 1023) / 1024, 64), batch), 256, 0, s>>>(
       dd, tau, C, S, reinterpret_cast<double2*>(U));
