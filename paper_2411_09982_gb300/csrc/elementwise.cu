@@ -253,7 +253,7 @@ __global__ void scale_minus_i_df_kernel(int per, const double* __restrict__ src,
   const double g = sq_dev ? __longlong_as_double((long long)(1023 - sq_dev[blockIdx.y]) << 52) : f;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < per; r += gridDim.x * blockDim.x) {
     const double2 v = reinterpret_cast<const double2*>(src)[base + r];
-    const df32 re = df_from_double(g * v.y), im = df_from_double(-g * v.x);
+    const df32 re = df_split(g * v.y), im = df_split(-g * v.x);
     dst[base + r] = make_float4(re.hi, re.lo, im.hi, im.lo);
   }
 }
@@ -495,7 +495,7 @@ __global__ void df_to_fp64_kernel(long long per, long long total, const float4* 
        e += (long long)gridDim.x * blockDim.x) {
     const long long b = e / per, r = e % per;
     const float4 v = src[b * ss + r];
-    dst[b * ds + r] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+    dst[b * ds + r] = make_double2(df_to_double(df32{v.x, v.y}), df_to_double(df32{v.z, v.w}));
   }
 }
 
@@ -505,7 +505,7 @@ __global__ void fp64_to_df_kernel(long long per, long long total, const double2*
        e += (long long)gridDim.x * blockDim.x) {
     const long long b = e / per, r = e % per;
     const double2 v = src[b * ss + r];
-    const df32 re = df_from_double(v.x), im = df_from_double(v.y);
+    const df32 re = df_split(v.x), im = df_split(v.y);
     dst[b * ds + r] = make_float4(re.hi, re.lo, im.hi, im.lo);
   }
 }

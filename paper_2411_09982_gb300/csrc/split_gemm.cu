@@ -180,11 +180,7 @@ __device__ __forceinline__ Pow2Pair pow2_pair(int k) {
 }
 // the scaled value as an exact pair of FP32 numbers
 __device__ __forceinline__ df32 scaled_pair(df32 a, Pow2Pair f) { return {(a.hi * f.f1) * f.f2, (a.lo * f.f1) * f.f2}; }
-__device__ __forceinline__ df32 scaled_pair(double a, Pow2Pair f) {
-  const float hi = __double2float_rn(a);
-  const float lo = __double2float_rn(a - (double)hi);
-  return {(hi * f.f1) * f.f2, (lo * f.f1) * f.f2};
-}
+__device__ __forceinline__ df32 scaled_pair(double a, Pow2Pair f) { return scaled_pair(df_split(a), f); }
 
 constexpr float kRoundMagic = 12582912.0f;   // 1.5 2^23
 __device__ __forceinline__ float round_to_int(float x) { return __fsub_rn(__fadd_rn(x, kRoundMagic), kRoundMagic); }
