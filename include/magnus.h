@@ -57,16 +57,16 @@ extern "C" {
 #define MG_EUNSUPPORTED -8   /* size or mode outside what the library supports     */
 
 /* ---- precision modes ------------------------------------------------------ */
-/* MG_PREC_FP64: FP64 operands and results throughout.  From d = 33 on the products of
- *   the exponential, of the propagators, of re-orthonormalisation and of the report run on
- *   the tcgen05 tensor cores from eight exact base-128 digits per operand (56 bits of
- *   every row's or column's largest entry, exact level sums, one FP64 rounding per entry);
- *   their error is below FP64 arithmetic's, relative to the largest entries of A's row and
- *   B's column.  Operands with a NaN, an infinity or a row or column scale outside
- *   2^-400 .. 2^400, smaller d and mg_cgemm take native FP64 arithmetic.  If a bounded
- *   device wait of such a product gives up, its outputs become NaN and the next call that
- *   reads the context's status returns MG_ETIMEOUT (the same call when it reports or
- *   copies to the host).
+/* MG_PREC_FP64: FP64 operands and results throughout.  From d = 33 on and where the batch is
+ *   large enough, the products of the exponential, of the propagators, of
+ *   re-orthonormalisation and of the report run on the tcgen05 tensor cores from eight
+ *   base-256 digits per operand (63 bits below every row's or column's largest entry, exact
+ *   level sums, one rounding per entry); their error is below FP64 arithmetic's, relative to
+ *   the largest entries of A's row and B's column.  Operands with a NaN, an infinity or a row
+ *   or column scale outside 2^-400 .. 2^400, small products and mg_cgemm take native FP64
+ *   arithmetic.  If a bounded device wait of a product on the tensor cores gives up, its
+ *   outputs become NaN and the next call that reads the context's status returns MG_ETIMEOUT
+ *   (the same call when it reports or copies to the host).
  * MG_PREC_SPLIT: matrix products on the tcgen05 tensor cores.  Each operand row
  *   (column) is scaled by a power of two and cut into `slices` signed BF16
  *   digits of `beta` bits; digit products are accumulated in FP32 TMEM

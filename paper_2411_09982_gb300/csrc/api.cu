@@ -355,12 +355,17 @@ int timing_mark(mg_ctx* ctx, int* idx) {
   return MG_OK;
 }
 
-// Smallest dimension whose FP64 products run from digits on the tensor cores.  Up to 32 the
-// FP64-pipe kernel covers a product with one 32 x 32 tile and is faster (exponentials of 512
-// matrices: d = 32 1.54 ms against 2.00 ms from digits); beyond, its 64 x 64 tiles pad the
-// FP64 work and the digits win at every batch (d = 40: 6.74 against 2.44 ms, one matrix 1.79
-// against 0.77 ms; d = 128: 79.9 against 7.7 ms).
+// FP64 products run from digits on the tensor cores (gemm_f64_digits.cu) from d = 33 on and
+// where the batch is worth it: from digits a small batch costs its slicers and one wave of
+// tiles however little work it is, on the FP64 pipe its work.  The two meet at dp^3 batch =
+// 6e6 to 1e7 (dp: d rounded up to the pipe kernel's 16-wide tiles) at every d; exponentials
+// from digits / on the pipe: one of d = 100 820 / 435 us, one of d = 200 1085 / 1200, 16 of
+// d = 64 600 / 449, 32 609 / 749, 128 751 / 2263, 8 of d = 128 882 / 1480.
 constexpr int kF64DigitsMinDim = 33;
+bool f64_digits_pay(int d, int batch) {
+  const long long dp = (d + 15) / 16 * 16;
+  return d >= kF64DigitsMinDim && dp * dp * dp * batch >= 8000000;
+}
 
 struct Engine {
   mg_ctx* ctx;
@@ -383,7 +388,8 @@ struct Engine {
   int sym = 0;                        // the next product's result is complex symmetric
   bool fp64_pipe = false;             // FP64 products on the FP64 pipe at every dimension (mg_cgemm)
   // FP64 products from integer digits on the tensor cores (gemm_f64_digits.cu)
-  bool digits64() const { return prec == MG_PREC_FP64 && !fp64_pipe && d >= kF64DigitsMinDim; }
+  bool digits64(int batch) const { return prec == MG_PREC_FP64 && !fp64_pipe && f64_digits_pay(d, batch); }
+  bool digits_dim() const { return prec == MG_PREC_FP64 && !fp64_pipe && d >= kF64DigitsMinDim; }   // some batch may
   bool allow18() const { return prec == MG_PREC_SPLIT && taylor_mode != MG_TAYLOR_PS; }
   SplitCtl ctl() const {
     SplitCtl c;
@@ -401,7 +407,7 @@ struct Engine {
   }
 
   int reserve(int batch) {
-    if (digits64()) {
+    if (digits64(batch)) {
       MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(d, batch), &abuf));
       MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(d, batch), &bbuf[0]));
       MG_TRY(ws_get(ctx, WS_BBUF1, f64d_b_bytes(d, batch), &bbuf[1]));
@@ -418,12 +424,12 @@ struct Engine {
   // the FP64 path stores FP64.  Both use 16 bytes per complex element.
   bool df() const { return prec == MG_PREC_SPLIT; }
   int prepA(int batch, const double* A, long long sA, int in_df) {
-    if (digits64()) return f64d_slice_a(d, batch, A, sA, 0, abuf, ctx->stream, ctl());
+    if (digits64(batch)) return f64d_slice_a(d, batch, A, sA, 0, abuf, ctx->stream, ctl());
     if (prec != MG_PREC_SPLIT) return MG_OK;
     return split_slice_a(d, L, batch, A, sA, in_df, abuf, ctx->stream, ctl());
   }
   int prepB(int slot, int batch, const double* B, long long sB, int in_df) {
-    if (digits64()) return f64d_slice_b(d, batch, B, sB, bbuf[slot], ctx->stream, ctl());
+    if (digits64(batch)) return f64d_slice_b(d, batch, B, sB, bbuf[slot], ctx->stream, ctl());
     if (prec != MG_PREC_SPLIT) return MG_OK;
     return split_slice_b(d, L, batch, B, sB, in_df, bbuf[slot], ctx->stream, ctl());
   }
@@ -441,7 +447,7 @@ struct Engine {
   // skipping never read (the zero half of A's K axis; the zero plane of B, or both -Im
   // and Im planes of a real B).  Otherwise the general slicers.
   int prep_poly(bool as_a, int slot, int batch, const double* M, int part) {
-    if (prec != MG_PREC_SPLIT && !digits64()) return MG_OK;
+    if (prec != MG_PREC_SPLIT && !digits64(batch)) return MG_OK;
     if (!lower()) {
       if (as_a) MG_TRY(prepA(batch, M, mat_doubles_(), 1));
       if (slot >= 0) MG_TRY(prepB(slot, batch, M, mat_doubles_(), 1));
@@ -504,7 +510,7 @@ struct Engine {
     if (prec == MG_PREC_SPLIT) {
       r = split_gemm(d, L, batch, abuf, bbuf[slot], C, sC, add, ctx->status, ctx->stream, ctl());
       a_zero = b_zero = sym = 0;
-    } else if (digits64()) {
+    } else if (digits64(batch)) {
       r = f64d_gemm(d, batch, 0, A, sA, abuf, B, sB, bbuf[slot], C, sC, add, ctx->slot_ptr[WS_F64_SUMS], ctx->sms,
                     ctx->status, ctx->stream, ctl());
     } else {
@@ -526,7 +532,7 @@ struct Engine {
   }
   int timing_begin(int* idx) { return timing_mark(ctx, idx); }
   // FP64 exponentials of real symmetric exponents from digits
-  bool real64() const { return digits64() && x_sym; }
+  bool real64(int batch) const { return digits64(batch) && x_sym; }
   // real products on the lower triangle that degree m and sq squarings take
   static int real_products(int m, int sq) {
     const int kc = m / 2, ks = (m - 1) / 2, p = (kc + 1) / 2;
@@ -766,7 +772,7 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
     if (sU != md) return MG_EINVAL;
     return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, tc.s, nullptr, U);
   }
-  if (eng.real64()) {
+  if (eng.real64(batch)) {
     if (sU != md) return MG_EINVAL;
     return eng.expm_real64(batch, W, tau, tc.m, tc.products, tc.s, nullptr, U);
   }
@@ -800,7 +806,7 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
                    const TaylorChoice& tc, int S, double* U, bool w_df) {
   PhaseRange range("expm");
   if (eng.small64()) return eng.expm_small(batch, W, tau, tc.m, tc.p, tc.products, S, sq_dev, U);
-  if (eng.real64()) return eng.expm_real64(batch, W, tau, tc.m, tc.products, S, sq_dev, U);
+  if (eng.real64(batch)) return eng.expm_real64(batch, W, tau, tc.m, tc.products, S, sq_dev, U);
   const long long md = mat_doubles(eng.d);
   MG_TRY(eng.scale_x(batch, W, W, 0, sq_dev, w_df));
   double *R, *Rn;
@@ -838,7 +844,7 @@ int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const
   const long long md = mat_doubles(eng.d);
   AddTerms none;
   Engine e{ctx, eng.d, MG_PREC_FP64, 0};
-  if (!e.digits64()) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
+  if (!e.digits64(batch)) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
   void *ab, *bb, *sums;
   MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, batch), &ab));
   MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(e.d, batch), &bb));
@@ -1768,8 +1774,8 @@ int fold_chunk(mg_ctx* ctx, Engine& eng, PropState& ps, int n, const double* U, 
     MG_TRY(ws(ctx, WS_VEC, 2 * d + 2, &tmp));
     if (!eng.df() && !ps.traj && reorth == 0 && d <= 64 && n >= 8) {
       // small d in FP64: the n dependent matrix-vector steps of the chain are
-      // latency-bound (1.7 us each at d = 30, 0.3 us at d = 2); while a level of the
-      // batched tree, which costs 32 us at d = 30 and 4 us at d = 2 however few products
+      // latency-bound (1.7 us each at d = 30, 0.4 us at d = 2); while a level of the
+      // batched tree, which costs 14 us at d = 30 and 7 us at d = 2 however few products
       // are left, halves more than 32 steps, it takes less time
       const int stop = 32;
       double* prods = const_cast<double*>(U);
@@ -1974,7 +1980,7 @@ int mg_evolve(mg_plan* p, int output, const double* in, double* out, int reorth_
     rep->max_norm1 = st.max_norm;
     rep->matrix_products = eng.products;
   }
-  if (p->precision == MG_PREC_SPLIT || (eng.digits64() && (rep || (flags & MG_FLAG_HOST_PTRS))))
+  if (p->precision == MG_PREC_SPLIT || (eng.digits_dim() && (rep || (flags & MG_FLAG_HOST_PTRS))))
     return check_status(ctx);
   if (flags & MG_FLAG_HOST_PTRS) MG_CUDA_TRY(cudaStreamSynchronize(s));
   return MG_OK;
@@ -3312,7 +3318,7 @@ void server_loop(mg_server* srv) {
     }
     ExpmStats st;
     if (fill > 0) rc = process_chunk(ctx, eng, segs, fill, 0, srv->segs_dev, srv->psi_dev, &st);
-    if (rc == MG_OK && (eng.prec == MG_PREC_SPLIT || eng.digits64())) rc = check_status(ctx);
+    if (rc == MG_OK && (eng.prec == MG_PREC_SPLIT || eng.digits_dim())) rc = check_status(ctx);
     // completed jobs leave; on an error every job of the group fails
     std::vector<SJob*> done_now;
     for (SJob* j : group)

@@ -1,7 +1,7 @@
 """FP64 products from digits on the tensor cores (csrc/gemm_f64_digits.cu).
 
-A two-interval propagator product U_1 U_0 (mg_propagate) is one such product from d = 33
-on.  It is held, against extended precision, to the bound of 56-bit operands (every entry
+A propagator product U_1 U_0 (mg_propagate) is one such product where the batch is large
+enough; the tests below fill it up with identities.  It is held, against extended precision, to the bound of 56-bit operands (every entry
 of a row or column rounded to 2^-56 of the power of two above its largest entry, digit
 products of level 9 and up dropped, the last level rounded to its own unit, the result
 rounded to FP64); the eight base-256 digits hold 63.
@@ -15,10 +15,16 @@ pytestmark = pytest.mark.gpu
 from paper_2411_09982_gb300 import magnus as M  # noqa: E402
 
 
-def product(ctx, A, B, more=()):
-    """A B (and the product with `more` later factors on the left) by mg_propagate."""
+def enough(d):
+    """A batch that takes the digits at dimension d."""
+    return 8000000 // (-(-d // 16) * 16) ** 3 + 1
+
+
+def product(ctx, A, B):
+    """A B by mg_propagate: the first of enough(d) pairs, the others identities (exact)."""
     d = A.shape[0]
-    U = torch.from_numpy(np.stack([B, A] + list(more))).cuda()
+    U = torch.eye(d, dtype=torch.complex128, device="cuda").repeat(2 * enough(d), 1, 1)
+    U[0], U[1] = torch.from_numpy(B).cuda(), torch.from_numpy(A).cuda()
     out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
     M.mg_propagate(ctx, U.shape[0], d, U, M.MG_OUT_PROPAGATOR, None, out, 0, M.MG_PREC_FP64)
     torch.cuda.synchronize()
@@ -79,7 +85,7 @@ def test_product_within_its_bound(d, kind):
         ctx.close()
 
 
-@pytest.mark.parametrize("d", [40, 150])
+@pytest.mark.parametrize("d", [209, 260])
 @pytest.mark.parametrize("case", ["nan_a", "inf_b", "out_of_range"])
 def test_operands_outside_the_digits_take_the_fp64_pipe(d, case):
     """NaN, infinities and exponents beyond 2^400 give what the FP64-pipe product gives, bit for bit."""
@@ -146,12 +152,15 @@ def test_real_symmetric_exponentials(d):
     try:
         for norm in (1e-9, 1e-5, 1e-2, 0.08, 0.3, 0.7, 3.0, 30.0):
             A = symmetric(rng, d, norm)
+            N = enough(d)
             plan = M.Plan(ctx, torch.from_numpy(A).cuda(), None, M.MG_PREC_FP64)
-            plan.set_controls(1, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((1, 1, 0), dtype=torch.float64))
+            plan.set_controls(N, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
             out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
             rep = plan.evolve(M.MG_OUT_PROPAGATOR, None, out)
-            # ~20 products of d-term sums, their errors doubled by every squaring (2^s <= 4 norm)
-            assert np.abs(out.cpu().numpy() - exact_exp(A)).max() <= 2.0 ** -53 * 20 * d * (1 + 4 * norm), (norm, rep)
+            # ~20 products of d-term sums, their errors doubled by every squaring (2^s <= 4 norm),
+            # in each of the N equal intervals
+            tol = N * 2.0 ** -53 * 20 * d * (1 + 4 * norm)
+            assert np.abs(out.cpu().numpy() - exact_exp(N * A)).max() <= tol, (norm, rep)
             plan.close()
     finally:
         ctx.close()
@@ -165,13 +174,13 @@ def test_batch_of_real_exponents_with_uneven_squarings():
         plans, outs = [], []
         for A in As:
             p = M.Plan(ctx, torch.from_numpy(A).cuda(), None, M.MG_PREC_FP64)
-            p.set_controls(2, 1, 0.0, 0.5, np.array([2.0]), torch.zeros((2, 1, 0), dtype=torch.float64))
+            p.set_controls(90, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((90, 1, 0), dtype=torch.float64))
             plans.append(p)
             outs.append(torch.empty(A.shape, dtype=torch.complex128, device="cuda"))
         assert M.mg_evolve_batch(ctx, plans, [M.MG_OUT_PROPAGATOR] * 5, [None] * 5, outs) == [0] * 5
         torch.cuda.synchronize()
         for A, o in zip(As, outs):
             norm = np.abs(A - np.trace(A) / len(A) * np.eye(len(A))).sum(0).max()
-            assert np.abs(o.cpu().numpy() - exact_exp(A)).max() <= 2.0 ** -53 * 20 * 80 * (1 + 4 * norm)
+            assert np.abs(o.cpu().numpy() - exact_exp(90 * A)).max() <= 90 * 2.0 ** -53 * 20 * 80 * (1 + 4 * norm)
     finally:
         ctx.close()
