@@ -508,7 +508,9 @@ int mg_cgemm_split_static(int device, void* stream, int batch, int d, const doub
  * action kernel of MG_FLAG_STATE_ACTION counts as one launch with 8 flops per
  * stored operator nonzero per operator application. */
 int mg_ctx_enable_gemm_timing(mg_ctx* ctx, int enable);
-/* Failure detection of the tensor-core product (MG_PREC_SPLIT).  Every wait of
+/* Failure detection of the tensor-core products (MG_PREC_SPLIT as described here; those of
+ * MG_PREC_FP64 take `seconds` for every wait before their own closing ones, and leave NaN in
+ * the outputs they do not finish).  Every wait of
  * its kernel on an mbarrier is bounded: a CTA that gives up records
  * MG_ETIMEOUT for the call and winds down without touching its outputs.  Only
  * the waits whose abandonment is safe take `seconds` (0 <= seconds <= 4; the
