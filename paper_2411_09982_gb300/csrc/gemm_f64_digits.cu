@@ -922,14 +922,15 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!*abort_flag) atomicExch(p.status, MG_DEV_TIMEOUT);
         *abort_flag = 1;
       }
-      // the tiles this CTA leaves unfinished are not left looking like a result
+      // the tiles this CTA leaves unfinished, marked items' among them, are not left looking
+      // like a result
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
       for (; t < tiles; t += gridDim.x) {
         const int b = (int)(t / per_item);
         int mt, nt;
         f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         const int row = mt * F8_BM + q * 32 + lane;
-        if (f8_skip(p, b) || row >= p.d) continue;
+        if ((p.item_sq && p.item_sq[b] <= p.sq_step) || row >= p.d) continue;
         const int n0 = nt * 4 * WC + c0;
         for (int c = n0; c < min(p.d, n0 + WC); ++c) {
           if constexpr (CPLX) reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
