@@ -29,8 +29,8 @@
 // transmon chain d = 81 2.7e-14 / 1.1e-13; transmon-resonator d = 80 1.1e-12 / 1.6e-12.
 // (Base-128 digits, 56 bits, need fewer drains but gave 2.3e-14, 1.3e-14, 1.0e-13, 1.1e-12.)
 // Operands that the scheme does not cover -- a NaN, an infinity, a row or column whose largest
-// entry lies outside 2^-400 .. 2^400 -- are marked by the slicers; the epilogue warps compute
-// such an item in FP64 arithmetic (f8_pipe_row).
+// entry lies outside 2^-400 .. 2^400 -- are marked by the slicers; such an item is computed in
+// FP64 arithmetic once a CTA's digit tiles are done (f8_pipe_items).
 //
 // Structure of the product kernel (persistent, one CTA of 640 threads per SM, 128 x 64
 // complex output tiles; every tile makes two sweeps over K, levels 4..7 first):
@@ -456,31 +456,65 @@ __device__ __forceinline__ bool f8_skip(const F8Args& p, int b) {
   return (p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.item_sq && p.item_sq[b] <= p.sq_step);
 }
 
-// One row's columns c0 .. c1 of a marked item in FP64 arithmetic, in the order of
-// cgemm_f64_kernel (the same bits).
-__device__ __noinline__ void f8_pipe_row(const F8Args& p, int b, int row, int c0, int c1) {
-  const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
-  const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
-  double2* C = reinterpret_cast<double2*>(p.C + b * p.sC);
-  for (int c = c0; c < c1; ++c) {
-    double re = 0.0, im = 0.0;
-    for (int k = 0; k < p.d; ++k) {
-      double2 x = p.opA ? A[(long long)k * p.d + row] : A[(long long)row * p.d + k];
-      if (p.opA) x.y = -x.y;
-      const double2 y = B[(long long)k * p.d + c];
-      re = fma(x.x, y.x, re);
-      re = fma(-x.y, y.y, re);
-      im = fma(x.x, y.y, im);
-      im = fma(x.y, y.x, im);
+__device__ __forceinline__ bool f8_pipe_item(const F8Args& p, int b) {
+  return (p.bad_a[b] | p.bad_b[b]) != 0 && !(p.item_sq && p.item_sq[b] <= p.sq_step);
+}
+
+// The marked items in FP64 arithmetic, once a CTA's digit tiles are done: no wait of theirs is
+// open then, however long this takes.  16 x 16 outputs per group of 256 threads (two groups:
+// the epilogue warps), dealt over all groups of the grid; operands through shared memory, sums
+// in the order of cgemm_f64_kernel (the same bits).
+__device__ __noinline__ void f8_pipe_items(const F8Args& p, double2* stage, int et) {
+  const int g = et >> 8, tx = et & 15, ty = (et >> 4) & 15, d = p.d;
+  double2* As = stage + g * (16 * 17 + 16 * 16);   // [k][i], pitch 17
+  double2* Bs = As + 16 * 17;                      // [k][j]
+  const int n = (d + 15) / 16, per = n * n;
+  const long long all = 2ll * gridDim.x;
+  long long turn = 2ll * blockIdx.x + g;           // tiles until this group's next one
+  auto sync = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); };
+  for (int b = 0; b < p.batch; ++b) {
+    if (!f8_pipe_item(p, b)) continue;
+    const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
+    const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
+    long long u = turn;
+    for (; u < per; u += all) {
+      const int i0 = (int)(u / n) * 16, j0 = (int)(u % n) * 16;
+      double re = 0.0, im = 0.0;
+      for (int k0 = 0; k0 < d; k0 += 16) {
+        double2 v = make_double2(0.0, 0.0), w = v;
+        if (p.opA == 0) {   // A[i0 + ty][k0 + tx]
+          if (i0 + ty < d && k0 + tx < d) v = A[(long long)(i0 + ty) * d + k0 + tx];
+          As[tx * 17 + ty] = v;
+        } else {            // conj(A[k0 + ty][i0 + tx])
+          if (i0 + tx < d && k0 + ty < d) v = A[(long long)(k0 + ty) * d + i0 + tx];
+          As[ty * 17 + tx] = make_double2(v.x, -v.y);
+        }
+        if (k0 + ty < d && j0 + tx < d) w = B[(long long)(k0 + ty) * d + j0 + tx];
+        Bs[ty * 16 + tx] = w;
+        sync();
+        const int kmax = min(16, d - k0);
+        for (int k = 0; k < kmax; ++k) {
+          const double2 x = As[k * 17 + ty], y = Bs[k * 16 + tx];
+          re = fma(x.x, y.x, re);
+          re = fma(-x.y, y.y, re);
+          im = fma(x.x, y.y, im);
+          im = fma(x.y, y.x, im);
+        }
+        sync();
+      }
+      const int i = i0 + ty, j = j0 + tx;
+      if (i < d && j < d) {
+        const long long off = (long long)i * d + j;
+        for (int m = 0; m < p.add_n; ++m) {
+          const double2 v = reinterpret_cast<const double2*>(p.add_src[m] + b * p.add_stride)[off];
+          re = fma(p.add_coef[m], v.x, re);
+          im = fma(p.add_coef[m], v.y, im);
+        }
+        if (i == j) re += p.diag;
+        reinterpret_cast<double2*>(p.C + b * p.sC)[off] = make_double2(re, im);
+      }
     }
-    const long long off = (long long)row * p.d + c;
-    for (int m = 0; m < p.add_n; ++m) {
-      const double2 v = reinterpret_cast<const double2*>(p.add_src[m] + b * p.add_stride)[off];
-      re = fma(p.add_coef[m], v.x, re);
-      im = fma(p.add_coef[m], v.y, im);
-    }
-    if (row == c) re += p.diag;
-    C[off] = make_double2(re, im);
+    turn = u - per;
   }
 }
 
@@ -585,6 +619,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   uint64_t* mmadone = accempty + 1;        // closing commit
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mmadone + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* marked_flag = abort_flag + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -596,6 +631,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     mbar_init(accempty, F8_EPI_WARPS);
     mbar_init(mmadone, 1);
     *abort_flag = 0;
+    *marked_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -746,6 +782,11 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       while (!mbar_try_wait(mmadone, 0) && global_ns() - t0 < 4000000000ull) {
       }
     }
+  } else if constexpr (CPLX) {
+    // ---------------- warps 2, 3: is any item marked? ----------------
+    bool any = false;
+    for (int b = threadIdx.x - 64; b < p.batch; b += 64) any |= f8_pipe_item(p, b);
+    if (any) *marked_flag = 1;
   }
   } else {
     // ---------------- epilogue (warps 4..19) ----------------
@@ -765,12 +806,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       int mt, nt;
       f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
       const int row0 = mt * F8_BM + q * 32, col0 = nt * 4 * WC + c0;
-      if (f8_skip(p, b)) {
-        if constexpr (CPLX)
-          if ((p.bad_a[b] | p.bad_b[b]) != 0 && !(p.item_sq && p.item_sq[b] <= p.sq_step) && row0 + lane < p.d)
-            f8_pipe_row(p, b, row0 + lane, col0, min(p.d, col0 + WC));
-        continue;
-      }
+      if (f8_skip(p, b)) continue;
       // uniform over the warp; a real tile's columns right of all its rows are not needed
       const bool live = row0 < p.d && col0 < p.d && (CPLX || col0 <= row0 + 31);
       long long acc[F8_VALS];
@@ -922,15 +958,15 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!*abort_flag) atomicExch(p.status, MG_DEV_TIMEOUT);
         *abort_flag = 1;
       }
-      // the tiles this CTA leaves unfinished, marked items' among them, are not left looking
-      // like a result
+      // the tiles this CTA leaves unfinished are not left looking like a result (marked items
+      // are computed below)
       const double nan = __longlong_as_double(0x7FF8000000000000ll);
       for (; t < tiles; t += gridDim.x) {
         const int b = (int)(t / per_item);
         int mt, nt;
         f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         const int row = mt * F8_BM + q * 32 + lane;
-        if ((p.item_sq && p.item_sq[b] <= p.sq_step) || row >= p.d) continue;
+        if (f8_skip(p, b) || row >= p.d) continue;
         const int n0 = nt * 4 * WC + c0;
         for (int c = n0; c < min(p.d, n0 + WC); ++c) {
           if constexpr (CPLX) reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
@@ -947,6 +983,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
+  if constexpr (CPLX)
+    if (warp >= 4 && *marked_flag) f8_pipe_items(p, staging, threadIdx.x - 128);
 }
 
 // ---------------------------------------------------------------------------
@@ -1046,8 +1084,9 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   p.sq_step = ctl.sq_step;
   p.stall = ctl.stall;
   p.wait_ns = std::min<unsigned long long>(ctl.wait_ns, 4000000000ull);
-  const long long tiles = (long long)p.ntn * p.ntm * batch;
-  const int grid = (int)std::min<long long>(tiles, sms);
+  // one CTA per tile up to one per SM, and no fewer than marked items' 16 x 16 tiles would fill
+  const long long tiles = (long long)p.ntn * p.ntm * batch, sub = ceil_div(d, 16);
+  const int grid = (int)std::min<long long>(std::max(tiles, (sub * sub * batch + 1) / 2), sms);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<true>), (int)smem));
   MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<true>)));

@@ -50,3 +50,21 @@ def test_unfinished_marked_items_do_not_keep_older_values():
         assert not stale.any(), int(stale.sum())
     finally:
         ctx.close()
+
+
+def test_marked_items_do_not_run_out_the_waits_of_the_others():
+    """A limit of 3 ms, no stall: marked items take their time on the FP64 pipe, and the other
+    items' products finish (their waits are for loads and products of their own)."""
+    rng = np.random.default_rng(1)
+    n, d = 6, 700
+    A = hermitian(rng, n, d, 1.5)
+    A[:2] *= 2.0 ** -450
+    ctx = M.Context(0)
+    try:
+        ctx.set_wait_limit(0.003)
+        U = expm(ctx, A)
+        assert np.abs(U[:2] - np.eye(d)).max() <= 1e-14
+        # ~10 products of d-term sums
+        assert np.abs(U[2:] - exact(A[2:])).max() <= 2.0 ** -53 * 20 * d
+    finally:
+        ctx.close()
