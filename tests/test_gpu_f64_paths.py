@@ -1,0 +1,79 @@
+"""MG_PREC_FP64 beside its results: the structure option, the counted work, the error of a product
+from digits at the 63 bits it holds, and per-interval squaring counts of complex operators."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2411_09982_gb300 import magnus as M  # noqa: E402
+
+
+def cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def enough(d):
+    return 8000000 // (-(-d // 16) * 16) ** 3 + 1
+
+
+def hermitian(rng, d, norm, real):
+    A = rng.normal(size=(d, d)) + (0 if real else 1j * rng.normal(size=(d, d)))
+    A = (A + A.conj().T).astype(np.complex128)
+    return A * (norm / np.abs(A - np.trace(A) / d * np.eye(d)).sum(0).max())
+
+
+def exact(A):
+    lam, V = np.linalg.eigh(A)
+    return (V * np.exp(-1j * lam)) @ V.conj().T
+
+
+def one_plan(ctx, A, N):
+    plan = M.Plan(ctx, cuda(A), None, M.MG_PREC_FP64)
+    plan.set_controls(N, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
+    return plan
+
+
+@pytest.mark.parametrize("d", [33, 64, 129, 300])
+def test_product_holds_63_bits(d):
+    """A product of Gaussian matrices against extended precision.  Rounding each entry to 2^-63 of
+    its row's or column's scale 2^E and leaving out the digit pairs s + t >= 8 (7 of them at
+    s + t = 8, digits of RMS 74) are random: sigma = sqrt(d) 2^-61 2^(Ea + Eb) for the sum over
+    2 d terms.  Eight of them (some 1e4 entries) beside the rounding of the result; without the
+    last digit the error would be 150 times sigma."""
+    rng = np.random.default_rng(d)
+    ctx = M.Context(0)
+    try:
+        A, B = (rng.normal(size=(d, d)) + 1j * rng.normal(size=(d, d)) for _ in range(2))
+        U = torch.eye(d, dtype=torch.complex128, device="cuda").repeat(2 * enough(d), 1, 1)
+        U[0], U[1] = cuda(B), cuda(A)
+        out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+        M.mg_propagate(ctx, U.shape[0], d, U, M.MG_OUT_PROPAGATOR, None, out, 0, M.MG_PREC_FP64)
+        C = out.cpu().numpy()
+        rows = np.unique(np.linspace(0, d - 1, 30).astype(int))
+        Ar, Ai, Br, Bi = (x.astype(np.longdouble) for x in (A.real[rows], A.imag[rows], B.real, B.imag))
+        re, im = Ar @ Br - Ai @ Bi, Ar @ Bi + Ai @ Br
+        scale = lambda x, axis: 2.0 ** (np.floor(np.log2(np.maximum(abs(x.real), abs(x.imag)).max(axis))) + 1)  # noqa: E731
+        sigma = np.sqrt(d) * 2.0 ** -61 * np.outer(scale(A, 1)[rows], scale(B, 0))
+        for ref, got in ((re, C.real[rows]), (im, C.imag[rows])):
+            assert np.all(np.abs((got - ref).astype(np.float64)) <= 2.0 ** -53 * np.abs(ref) + 8 * sigma)
+    finally:
+        ctx.close()
+
+
+def test_batch_of_complex_exponents_with_uneven_squarings():
+    """Per-interval squaring counts, complex products from digits (d > 32)."""
+    rng = np.random.default_rng(11)
+    N = 90
+    ctx = M.Context(0)
+    try:
+        As = [hermitian(rng, d, norm, False) for d, norm in ((40, 0.1), (45, 40.0), (48, 2.0), (70, 5.0), (33, 1e-3))]
+        plans = [one_plan(ctx, A, N) for A in As]
+        outs = [torch.empty(A.shape, dtype=torch.complex128, device="cuda") for A in As]
+        assert M.mg_evolve_batch(ctx, plans, [M.MG_OUT_PROPAGATOR] * 5, [None] * 5, outs) == [0] * 5
+        for A, o in zip(As, outs):
+            norm = np.abs(A - np.trace(A) / len(A) * np.eye(len(A))).sum(0).max()
+            # N intervals of ~20 products of d-term sums, doubled by every squaring
+            assert np.abs(o.cpu().numpy() - exact(N * A)).max() <= N * 2.0 ** -53 * 20 * 80 * (1 + 4 * norm)
+    finally:
+        ctx.close()
