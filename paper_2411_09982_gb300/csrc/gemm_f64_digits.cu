@@ -122,10 +122,10 @@ size_t f64d_b_bytes(int d, int batch) {
 // ---------------------------------------------------------------------------
 // slicers
 // ---------------------------------------------------------------------------
-// E with |a| < 2^E; zero and subnormals -> -2^29; NaN and infinities -> 1025
+// E with |a| < 2^E; zero -> -2^29; subnormals -> -1022; NaN and infinities -> 1025
 __device__ __forceinline__ int f8_exp(double a) {
-  const int bexp = (__double2hiint(a) >> 20) & 0x7FF;
-  return bexp == 0 ? -(1 << 29) : bexp - 1022;
+  const int hi = __double2hiint(a), bexp = (hi >> 20) & 0x7FF;
+  return bexp == 0 ? ((((uint32_t)hi << 1) | (uint32_t)__double2loint(a)) ? -1022 : -(1 << 29)) : bexp - 1022;
 }
 // exponents are stored as E + 4096; 0 is a row or column without a nonzero entry
 constexpr int F8_EBIAS = 4096;
@@ -138,12 +138,11 @@ constexpr unsigned long long F8_BIAS = 0x8080808080808080ull;   // 128 in every 
 __device__ __forceinline__ unsigned long long f8_fixed(double a, int E) {
   const long long bits = __double_as_longlong(a);
   const int bexp = (int)((bits >> 52) & 0x7FF);
-  const int sh = bexp - 1075 + 62 - E;                       // <= 9
-  unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  if (sh >= 0) m <<= min(sh, 9);
+  const int sh = max(bexp, 1) - 1075 + 62 - E;               // <= 9, 10 for subnormals
+  unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(bexp != 0) << 52);
+  if (sh >= 0) m <<= min(sh, 10);
   else if (sh > -56) m = (m + (1ull << (-sh - 1))) >> -sh;
   else m = 0;
-  if (bexp == 0) m = 0;                                      // zero (a subnormal is below any kept bit)
   return (bits < 0 ? 0ull - m : m) + F8_BIAS;
 }
 // q_s 2^{-8 s} of a biased value as FP32 (exact): the byte in the low mantissa bits of
@@ -335,8 +334,8 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
 // Row digits of a real symmetric matrix (both operands of its products are such rows), one
 // warp per row: entry k is X[k] + sz Z[k] (Z null: X[k]), or with CW the real part of a complex
 // matrix W times 2^{-sq} (an exact change of the row's exponent).  grid (ceil(d / 8), batch).
-// Entries are bounded (the exponential scales them to norm about 1); rows below 2^-400 are
-// rounded at that scale, far below anything the result holds.
+// Entries are bounded above (the exponential scales them to norm about 1) and finite, so no
+// row is marked; the product takes scales down to the smallest subnormal (f8_value_any).
 template <bool CW>
 __global__ void __launch_bounds__(256)
 f64r_slice_kernel(int d, int Kh, const double* __restrict__ X, const double* __restrict__ Z, double sz, long long sX,
@@ -356,7 +355,6 @@ f64r_slice_kernel(int d, int Kh, const double* __restrict__ X, const double* __r
   for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   const int s = CW ? (sq_dev ? sq_dev[b] : sq) : 0;
   if (E < -(1 << 28)) E = s;                 // all-zero row
-  E = max(E, s - F8_EXP_MAX);
   if (lane == 0) ex[(long long)b * d + row] = E - s + F8_EBIAS;
   __nv_bfloat16* o = out + b * item_elems + (long long)row * Kh;
   const long long ds = (long long)d * Kh;
@@ -559,6 +557,14 @@ __device__ __forceinline__ double f8_value_fp64(long long t, uint32_t w, int k) 
   const double h = __longlong_as_double(t + 0x4338000000000000ll) - 6755399441055744.0;   // (1.5 2^52 + t) - 1.5 2^52
   const double l = __hiloint2double(0x43300000, (int)w) - 4503599627370496.0;             // (2^52 + w) - 2^52
   return fma(h, 4294967296.0, l) * __hiloint2double((k + 1023) << 20, 0);
+}
+
+// Either of the two for any k: real rows may be scaled down to the smallest subnormal.
+template <bool PIPE>
+__device__ __forceinline__ double f8_value_any(long long t, uint32_t w, int k) {
+  const bool tiny = k < -1000;
+  const double x = PIPE ? f8_value_fp64(t, w, tiny ? -60 : k) : f8_value(t, w, tiny ? -60 : k);
+  return tiny ? scalbn(x, k + 60) : x;
 }
 
 // Drain of one accumulator set (levels l0 .. l0 + 3) into the thread's sums, in units of
@@ -873,7 +879,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int v = 0; v < 8; ++v) {
               const int col = col0 + c + v;
               const int k = Ea + (col < p.d ? f8_exponent(ebp[col]) : 0) - 68 + p.scale2;
-              double x = v % 4 == 3 ? f8_value_fp64(acc[c + v], w[v], k) : f8_value(acc[c + v], w[v], k);
+              double x = v % 4 == 3 ? f8_value_any<true>(acc[c + v], w[v], k) : f8_value_any<false>(acc[c + v], w[v], k);
               if (row < p.d && col <= row) {
                 const long long off = (long long)col * p.d + row;
 #pragma unroll

@@ -68,3 +68,54 @@ def test_marked_items_do_not_run_out_the_waits_of_the_others():
         assert np.abs(U[2:] - exact(A[2:])).max() <= 2.0 ** -53 * 20 * d
     finally:
         ctx.close()
+
+
+def test_subnormal_rows_and_columns_take_fp64_arithmetic():
+    """A row of A (a column of B) with nothing but subnormal entries is not a zero one."""
+    rng = np.random.default_rng(2)
+    d = 64
+    n = 8000000 // d ** 3 + 1
+    ctx = M.Context(0)
+    try:
+        for side in (0, 1):
+            A, B = (rng.normal(size=(2, d, d)) + 1j * rng.normal(size=(2, d, d)))
+            if side == 0:
+                A[5] *= 2.0 ** -1060
+                B *= 2.0 ** 300
+            else:
+                B[:, 5] *= 2.0 ** -1060
+                A *= 2.0 ** 300
+            U = torch.eye(d, dtype=torch.complex128, device="cuda").repeat(2 * n, 1, 1)
+            U[0], U[1] = torch.from_numpy(B).cuda(), torch.from_numpy(A).cuda()
+            out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+            M.mg_propagate(ctx, 2 * n, d, U, M.MG_OUT_PROPAGATOR, None, out, 0, M.MG_PREC_FP64)
+            ref = torch.empty((1, d, d), dtype=torch.complex128, device="cuda")
+            M.mg_cgemm(ctx, 1, d, U[1:2].contiguous(), U[0:1].contiguous(), ref, M.MG_PREC_FP64)
+            torch.cuda.synchronize()
+            assert torch.equal(torch.view_as_real(out), torch.view_as_real(ref[0]))
+            assert (ref[0].abs() > 0).all()
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("d", [33, 130])
+def test_tiny_real_symmetric_exponents_keep_their_bits(d):
+    """exp(-i A) of a real symmetric A of 2^-450: entry by entry I - i A."""
+    rng = np.random.default_rng(3)
+    n = 8000000 // (-(-d // 16) * 16) ** 3 + 1
+    A = rng.normal(size=(d, d))
+    A = (A + A.T) * 2.0 ** -450
+    ctx = M.Context(0)
+    try:
+        plan = M.Plan(ctx, torch.from_numpy(A.astype(np.complex128)).cuda(), None, M.MG_PREC_FP64)
+        plan.set_controls(n, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((n, 1, 0), dtype=torch.float64))
+        psi = np.zeros(d, dtype=np.complex128)
+        psi[3] = 1.0
+        traj = torch.empty((n + 1, d), dtype=torch.complex128, device="cuda")
+        plan.evolve(M.MG_OUT_TRAJECTORY, torch.from_numpy(psi).cuda(), traj)
+        got = traj[1].cpu().numpy()
+        off = np.arange(d) != 3
+        assert np.abs(got[off].imag + A[off, 3]).max() <= 1e-14 * np.abs(A).max()
+        plan.close()
+    finally:
+        ctx.close()
