@@ -62,11 +62,16 @@ extern "C" {
  *   re-orthonormalisation and of the report run on the tcgen05 tensor cores from eight
  *   base-256 digits per operand (63 bits below every row's or column's largest entry, exact
  *   level sums, one rounding per entry); their error is below FP64 arithmetic's, relative to
- *   the largest entries of A's row and B's column.  Operands with a NaN, an infinity or a row
- *   or column scale outside 2^-400 .. 2^400, small products and mg_cgemm take native FP64
- *   arithmetic.  If a bounded device wait of a product on the tensor cores gives up, its
- *   outputs become NaN and the next call that reads the context's status returns MG_ETIMEOUT
- *   (the same call when it reports or copies to the host).
+ *   the largest entries of A's row and B's column: in a propagator, an amplitude 2^-k below
+ *   the largest of its row holds about 60 - k bits (FP64 arithmetic 53 whatever k).  Where the
+ *   operands are the caller's -- mg_expm, mg_propagate, the running product of an evolution
+ *   resumed from `in` -- every entry holds FP64 arithmetic's bound, about
+ *   d 2^-53 sum_k |a_ik| |b_kj|: 128 x 64 blocks with weaker entries than the digits hold so
+ *   take native FP64 arithmetic, 2 to 20 times slower.  So do operands with a NaN, an
+ *   infinity or a row or column scale outside 2^-400 .. 2^400, small products and mg_cgemm.
+ *   If a bounded device wait of a product on the tensor cores gives up, its outputs become
+ *   NaN and the next call that reads the context's status returns MG_ETIMEOUT (the same call
+ *   when it reports or copies to the host).
  * MG_PREC_SPLIT: matrix products on the tcgen05 tensor cores.  Each operand row
  *   (column) is scaled by a power of two and cut into `slices` signed BF16
  *   digits of `beta` bits; digit products are accumulated in FP32 TMEM

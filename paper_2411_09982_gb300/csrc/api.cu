@@ -387,6 +387,9 @@ struct Engine {
   int a_zero = 0, b_zero = 0;         // structure of the next product's operands
   int sym = 0;                        // the next product's result is complex symmetric
   bool fp64_pipe = false;             // FP64 products on the FP64 pipe at every dimension (mg_cgemm)
+  // operands of the next products are a caller's own, of any range of magnitudes: FP64's error
+  // bound entry by entry (products from digits check for it)
+  bool entrywise = false;
   // FP64 products from integer digits on the tensor cores (gemm_f64_digits.cu)
   bool digits64(int batch) const { return prec == MG_PREC_FP64 && !fp64_pipe && f64_digits_pay(d, batch); }
   bool digits_dim() const { return prec == MG_PREC_FP64 && !fp64_pipe && d >= kF64DigitsMinDim; }   // some batch may
@@ -412,7 +415,7 @@ struct Engine {
       MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(d, batch), &bbuf[0]));
       MG_TRY(ws_get(ctx, WS_BBUF1, f64d_b_bytes(d, batch), &bbuf[1]));
       void* sums;
-      return ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms), &sums);
+      return ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms, d, batch), &sums);
     }
     if (prec != MG_PREC_SPLIT) return MG_OK;
     MG_TRY(ws_get(ctx, WS_ABUF, split_a_bytes(d, L, batch), &abuf));
@@ -512,7 +515,7 @@ struct Engine {
       a_zero = b_zero = sym = 0;
     } else if (digits64(batch)) {
       r = f64d_gemm(d, batch, 0, A, sA, abuf, B, sB, bbuf[slot], C, sC, add, ctx->slot_ptr[WS_F64_SUMS], ctx->sms,
-                    ctx->status, ctx->stream, ctl());
+                    entrywise, ctx->status, ctx->stream, ctl());
     } else {
       AddTerms a = add;
       a.item_sq = item_sq;
@@ -599,6 +602,14 @@ struct Engine {
   }
 };
 
+// Products within its scope take operands of any range of magnitudes (`on`).
+struct Entrywise {
+  Engine& eng;
+  const bool before;
+  Entrywise(Engine& e, bool on) : eng(e), before(e.entrywise) { e.entrywise = before || on; }
+  ~Entrywise() { eng.entrywise = before; }
+};
+
 long long mat_doubles(int d) { return 2LL * d * d; }
 
 // ---------------------------------------------------------------------------
@@ -613,9 +624,9 @@ struct ExpmStats {
 // Taylor polynomial T_m(X) of a batch (degree tc.m; p = 0: the five-product degree-18
 // scheme, else Paterson-Stockmeyer with block size p).  X = W (engine storage) is
 // overwritten where the scheme reuses it.  *R receives the result, *Rn the other
-// Horner buffer (free for the squarings).
+// Horner buffer (free for the squarings).  less_identity (not with p = 0): T_m(X) - I.
 int taylor_poly(mg_ctx* ctx, Engine& eng, int batch, double* W, const TaylorChoice& tc, double** R_out,
-                double** Rn_out) {
+                double** Rn_out, bool less_identity = false) {
   const int d = eng.d;
   const long long md = mat_doubles(d);
   double *P2, *P3, *Y, *R0, *R1;
@@ -684,6 +695,7 @@ int taylor_poly(mg_ctx* ctx, Engine& eng, int batch, double* W, const TaylorChoi
   a[0] = 1.0;
   for (int j = 1; j <= 16; ++j) a[j] = a[j - 1] / j;
   auto coef = [&](int j) { return j <= tc.m ? a[j] : 0.0; };
+  auto diag_of = [&](int block) { return block == 0 && less_identity ? 0.0 : coef(block * tc.p); };
 
   // powers P_1 = X, ..., P_p = Y
   const int p = tc.p, m = tc.m;
@@ -707,7 +719,7 @@ int taylor_poly(mg_ctx* ctx, Engine& eng, int batch, double* W, const TaylorChoi
     int ns = 0;
     int top = (r == 0) ? q - 1 : q;
     for (int j = 1; j < p; ++j) { src[ns] = P[j]; cf[ns] = coef(top * p + j); ++ns; }
-    double diag = coef(top * p);
+    double diag = diag_of(top);
     if (r == 0) { src[ns] = P[p]; cf[ns] = coef(m); ++ns; }
     MG_TRY(eng.lincomb(batch, R, ns, src, cf, diag));
     i_next = top - 1;
@@ -718,7 +730,7 @@ int taylor_poly(mg_ctx* ctx, Engine& eng, int batch, double* W, const TaylorChoi
     add.n = 0;
     for (int j = 1; j < p; ++j) { add.src[add.n] = P[j]; add.coef[add.n] = coef(i * p + j); ++add.n; }
     add.stride = md;
-    add.diag = coef(i * p);
+    add.diag = diag_of(i);
     MG_TRY(eng.prep_poly(true, -1, batch, R, 0));
     eng.set_sym();
     MG_TRY(eng.mul(batch, R, md, 1, P[p], md, Rn, md, add));
@@ -779,13 +791,32 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
   // X = -i 2^{-s} W   (in place, into the engine's storage format)
   MG_TRY(eng.scale_x(batch, W, W, tc.s, nullptr, w_df));
   double *R, *Rn;
-  MG_TRY(taylor_poly(ctx, eng, batch, W, tc, &R, &Rn));
+  // Arbitrary operands from digits: the squarings run on E = T_m(X) - I, E' = E E + 2 E.  T
+  // itself has weak entries beside a diagonal of ones where X is small (a batch of norms 0.1 to
+  // 20 squares all of its items as often as the largest), which the digits do not hold to
+  // FP64's bound: 64 dense matrices of d = 81 took FP64 arithmetic in many tiles, 3.9 ms
+  // against 1.5 on E, whose entries are of one size.  (1.2 without the check of the products;
+  // relative error 9e-15 unchecked on T, 2.9e-15 so.)
+  const bool less_identity = eng.entrywise && eng.digits64(batch);
+  MG_TRY(taylor_poly(ctx, eng, batch, W, tc, &R, &Rn, less_identity));
   // squarings
   for (int k = 0; k < tc.s; ++k) {
     MG_TRY(eng.prep_poly(true, 0, batch, R, 0));
-    AddTerms none;
+    AddTerms add;
+    if (less_identity) {
+      add.n = 1;
+      add.src[0] = R;
+      add.coef[0] = 2.0;
+      add.stride = md;
+    }
     eng.set_sym();
-    MG_TRY(eng.mul(batch, R, md, 0, R, md, Rn, md, none));
+    MG_TRY(eng.mul(batch, R, md, 0, R, md, Rn, md, add));
+    std::swap(R, Rn);
+  }
+  if (less_identity) {
+    const double* src[1] = {R};
+    const double one[1] = {1.0};
+    MG_TRY(eng.lincomb(batch, Rn, 1, src, one, 1.0));
     std::swap(R, Rn);
   }
   // exact trace phase e^{-i tau_b}
@@ -839,7 +870,9 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
 }
 
 // C = opA(A) B in FP64 (report and re-orthonormalisation products): from digits where the
-// engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`.
+// engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`.  Entry
+// by entry only where the engine's products are FP64 ones (split states carry larger errors,
+// and the report takes the largest entry of its product).
 int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const double* B, double* C) {
   const long long md = mat_doubles(eng.d);
   AddTerms none;
@@ -848,13 +881,14 @@ int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const
   void *ab, *bb, *sums;
   MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, batch), &ab));
   MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(e.d, batch), &bb));
-  MG_TRY(ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms), &sums));
+  MG_TRY(ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms, e.d, batch), &sums));
   if (eng.abuf) eng.abuf = ab;   // the slots may have grown
   if (eng.bbuf[0]) eng.bbuf[0] = bb;
   const SplitCtl c = e.ctl();
   MG_TRY(f64d_slice_a(e.d, batch, A, md, opA, ab, ctx->stream, c));
   MG_TRY(f64d_slice_b(e.d, batch, B, md, bb, ctx->stream, c));
-  return f64d_gemm(e.d, batch, opA, A, md, ab, B, md, bb, C, md, none, sums, ctx->sms, ctx->status, ctx->stream, c);
+  return f64d_gemm(e.d, batch, opA, A, md, ab, B, md, bb, C, md, none, sums, ctx->sms, eng.entrywise && !eng.df(),
+                  ctx->status, ctx->stream, c);
 }
 
 // One Newton-Schulz polar step in FP64 on a batch: Z <- Z (3I - Z^dag Z)/2.
@@ -1721,6 +1755,7 @@ int mg_expm(mg_ctx* ctx, int batch, int d, const double* A, double* U, int preci
   MG_TRY(validate_prec(precision, slices));
   MG_CUDA_TRY(cudaSetDevice(ctx->device));
   Engine eng{ctx, d, precision, slices};
+  eng.entrywise = true;   // any Hermitian A
   const long long md = mat_doubles(d);
   const int chunk = chunk_size(ctx, d, precision, slices, batch, 1);
   for (int b0 = 0; b0 < batch; b0 += chunk) {
@@ -1761,6 +1796,7 @@ struct PropState {
   double* psi = nullptr;     // state mode (device, workspace)
   double* acc = nullptr;     // propagator mode: running product (device, workspace)
   bool acc_init = false;
+  bool resumed = false;      // acc began as the caller's matrix
   int done = 0;
 };
 
@@ -1814,11 +1850,15 @@ int fold_chunk(mg_ctx* ctx, Engine& eng, PropState& ps, int n, const double* U, 
     MG_TRY(eng.prepA(1, chunk_prod, md));
     MG_TRY(eng.prepB(0, 1, ps.acc, md));
     AddTerms none;
+    Entrywise any(eng, ps.resumed);
     MG_TRY(eng.mul(1, chunk_prod, md, 0, ps.acc, md, acc2, md, none));
     MG_TRY(launch_copy_strided(1, md, acc2, md, ps.acc, md, ctx->stream));
   }
   ps.done += n;
-  if (reorth > 0 && (ps.done / reorth) != ((ps.done - n) / reorth)) MG_TRY(reorth_batch(ctx, eng, 1, ps.acc, md));
+  if (reorth > 0 && (ps.done / reorth) != ((ps.done - n) / reorth)) {
+    Entrywise any(eng, ps.resumed);
+    MG_TRY(reorth_batch(ctx, eng, 1, ps.acc, md));
+  }
   return MG_OK;
 }
 
@@ -1849,7 +1889,7 @@ int begin_prop(mg_ctx* ctx, Engine& eng, PropState& ps, const double* in, int fl
       MG_TRY(ws(ctx, WS_OUT, md, &t));
       MG_CUDA_TRY(cudaMemcpyAsync(t, in, sizeof(double) * md, kind, ctx->stream));
       MG_TRY(eng.from_fp64(1, t, md, ps.acc, md));
-      ps.acc_init = true;
+      ps.acc_init = ps.resumed = true;
     }
   }
   return MG_OK;
@@ -1993,6 +2033,7 @@ int mg_propagate(mg_ctx* ctx, int N, int d, const double* U, int output, const d
   MG_TRY(validate_prec(precision, slices));
   MG_CUDA_TRY(cudaSetDevice(ctx->device));
   Engine eng{ctx, d, precision, slices};
+  eng.entrywise = true;   // any U
   PropState ps;
   ps.output = output;
   ps.d = d;
@@ -2032,6 +2073,7 @@ struct BatchJob {
   const double* c = nullptr;   // quadrature coefficients N x K (device)
   double* state = nullptr;     // padded psi (dp) or running product (dp x dp, engine storage)
   bool init = false;
+  bool resumed = false;        // the running product began as the caller's matrix
   bool failed = false;
   int done = 0;                // intervals applied so far
 };
@@ -2092,6 +2134,7 @@ int process_chunk(mg_ctx* ctx, Engine& eng, std::vector<ChunkSeg>& segs, int fil
       if (reorth_every > 1) { span = 1; while (span * 2 <= reorth_every) span *= 2; if (span < 2) span = 0; }
       double* prod;
       MG_TRY(tree_product(ctx, eng, g.n, Ub + g.off * md, &prod, span));
+      Entrywise any(eng, j.resumed);
       if (!j.init) {
         MG_TRY(launch_copy_strided(1, md, prod, md, j.state, md, s));
         j.init = true;
@@ -2250,7 +2293,7 @@ int init_job_state(mg_ctx* ctx, Engine& eng, BatchJob& j, const double* in, cuda
     MG_TRY(launch_identity(1, dp, tp, s));
     MG_TRY(launch_pad_into(d, dp, t, tp, s));
     MG_TRY(eng.from_fp64(1, tp, md, j.state, md));
-    j.init = true;
+    j.init = j.resumed = true;
   }
   return MG_OK;
 }
@@ -2555,6 +2598,7 @@ int issue_chunk(mg_ctx* ctx, Engine& eng, GroupProgram& G, ChunkPlan& ch) {
     if (G.reorth > 1) { span = 1; while (span * 2 <= G.reorth) span *= 2; if (span < 2) span = 0; }
     double* prod;
     MG_TRY(tree_product(ctx, eng, g.n, Ub + g.off * md, &prod, span));
+    Entrywise any(eng, j.resumed);
     if (!j.init) {
       MG_TRY(launch_copy_strided(1, md, prod, md, j.state, md, s));
       j.init = true;
@@ -2669,7 +2713,7 @@ int issue_group(mg_ctx* ctx, GroupProgram& G, const double* const* in, double* c
   MG_CUDA_TRY(cudaMemsetAsync(G.job_fail, 0, sizeof(int) * G.jobs.size(), s));
   MG_CUDA_TRY(cudaMemsetAsync(G.overflow, 0, sizeof(int), s));
   for (BatchJob& j : G.jobs) {
-    j.init = false;
+    j.init = j.resumed = false;
     j.done = 0;
     MG_TRY(init_job_state(ctx, eng, j, in ? in[j.idx] : nullptr, h2d, s));
   }

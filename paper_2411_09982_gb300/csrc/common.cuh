@@ -183,17 +183,19 @@ int split_gemm(int d, int L, int batch, const void* abuf, const void* bbuf, doub
 // FP64 products from integer digits on the tensor cores; see gemm_f64_digits.cu.  Operand
 // buffers are filled by the slicers (opA: 0 = A, 1 = A^dagger); the product also takes the
 // operands themselves, for items the slicers marked as outside the digits' range, so C
-// must not alias them.  scratch: f64d_scratch_bytes(sms) of device memory.
+// must not alias them.  entrywise: tiles with entries that the digits do not hold to FP64's
+// error bound, entry by entry, run in FP64 arithmetic (operands of any range of magnitudes).
+// scratch: f64d_scratch_bytes of device memory.
 size_t f64d_a_bytes(int d, int batch);
 size_t f64d_b_bytes(int d, int batch);
-size_t f64d_scratch_bytes(int sms);
+size_t f64d_scratch_bytes(int sms, int d, int batch);
 int f64d_slice_a(int d, int batch, const double* A, long long sA, int opA, void* buf, cudaStream_t s,
                  const SplitCtl& ctl = SplitCtl());
 int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cudaStream_t s,
                  const SplitCtl& ctl = SplitCtl());
 int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const void* abuf, const double* B,
               long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
-              int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
+              bool entrywise, int* status, cudaStream_t s, const SplitCtl& ctl = SplitCtl());
 
 // FP64 exponentials of real symmetric exponents from digits (cosine and sine, real symmetric
 // products); see f64r_expm.

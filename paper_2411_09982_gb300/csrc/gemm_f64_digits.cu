@@ -30,7 +30,8 @@
 // (Base-128 digits, 56 bits, need fewer drains but gave 2.3e-14, 1.3e-14, 1.0e-13, 1.1e-12.)
 // Operands that the scheme does not cover -- a NaN, an infinity, a row or column whose largest
 // entry lies outside 2^-400 .. 2^400 -- are marked by the slicers; such an item is computed in
-// FP64 arithmetic once a CTA's digit tiles are done (f8_pipe_items).
+// FP64 arithmetic once a CTA's digit tiles are done (f8_pipe_tiles).  So are, where a caller's own
+// operands are multiplied, tiles with entries too weak for the digits (f64d_weak_kernel).
 //
 // Structure of the product kernel (persistent, one CTA of 640 threads per SM, 128 x 64
 // complex output tiles; every tile makes two sweeps over K, levels 4..7 first):
@@ -432,6 +433,7 @@ struct F8Args {
   const int* eb;
   const int* bad_a;
   const int* bad_b;
+  const unsigned char* weak;  // per tile: the digits do not hold its weakest entries (null: not asked)
   const uint32_t* en_a;       // per item: largest digit energies of a K step (f8_energy)
   const uint32_t* en_b;
   double* C;
@@ -450,69 +452,194 @@ struct F8Args {
   int stall;                  // test only: the MMA issuer waits on a barrier nothing completes
 };
 
-__device__ __forceinline__ bool f8_skip(const F8Args& p, int b) {
-  return (p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.item_sq && p.item_sq[b] <= p.sq_step);
+__device__ __forceinline__ bool f8_done(const F8Args& p, int b) { return p.item_sq && p.item_sq[b] <= p.sq_step; }
+// tile t (of item b) runs in FP64 arithmetic
+__device__ __forceinline__ bool f8_pipe_tile(const F8Args& p, int b, long long t) {
+  return ((p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.weak && p.weak[t])) && !f8_done(p, b);
+}
+__device__ __forceinline__ bool f8_skip(const F8Args& p, int b, long long t) {
+  return (p.bad_a && (p.bad_a[b] | p.bad_b[b]) != 0) || (p.weak && p.weak[t]) || f8_done(p, b);
 }
 
-__device__ __forceinline__ bool f8_pipe_item(const F8Args& p, int b) {
-  return (p.bad_a[b] | p.bad_b[b]) != 0 && !(p.item_sq && p.item_sq[b] <= p.sq_step);
+// Where the operands are a caller's own (any range of magnitudes in a row), FP64 arithmetic
+// bounds the error of an entry by about d u M_ij + u |P_ij|, M = |A| |B| and P the addends; the
+// digits' is sqrt(d) 2^-61 2^{Ea_i + Eb_j} whatever the entry's own terms are (the standard
+// deviation of rounding each entry at 2^-63 of its row's or column's scale and of leaving out
+// the digit pairs s + t >= 8).  This kernel forms M in FP32 (the larger component's magnitude,
+// rounded down, scaled by 2^{57 - Ea}, 2^{57 - Eb}) and sends a tile to FP64 arithmetic where
+// an entry has M + |P| / d < 2^{114 - 8} / sqrt(d).  M = 0 is a zero of the operands'
+// structure, which the digits give exactly, unless some entry in reach is below 2^-110 of its
+// row or column.  128 x 64 outputs per CTA (the product's tiles), 4 x 4 per thread; small d is
+// bound by latency: d = 81, batch 64 takes 16 us a product (256 threads of 8 x 4 outputs: 42).
+constexpr int F8_NK = 16;              // K per slab
+constexpr int F8_WEAK_THREADS = 512;
+// the larger component's magnitude times 2^k, rounded down (0 below FP32's normal range,
+// infinity above it); without FP64 instructions
+__device__ __forceinline__ float f8_magnitude(double2 v, int k) {
+  const int hi = max(__double2hiint(v.x) & 0x7FFFFFFF, __double2hiint(v.y) & 0x7FFFFFFF);
+  const int fe = (hi >> 20) - 1023 + 127 + k;
+  if (hi < 0x00100000 || fe <= 0) return 0.f;
+  return fe >= 255 ? __int_as_float(0x7F800000) : __int_as_float((fe << 23) | ((hi & 0xFFFFF) << 3));
+}
+__device__ __forceinline__ bool f8_nonzero(double2 v) {
+  return (((unsigned long long)__double_as_longlong(v.x) | (unsigned long long)__double_as_longlong(v.y)) << 1) != 0;
+}
+__global__ void __launch_bounds__(F8_WEAK_THREADS)
+f64d_weak_kernel(const __grid_constant__ F8Args p, float least, unsigned char* __restrict__ weak) {
+  __shared__ __align__(16) float As[F8_NK][F8_BM + 4], Bs[F8_NK][F8_BN];
+  const int b = blockIdx.y, tid = threadIdx.x, d = p.d;
+  const long long t = (long long)b * gridDim.x + blockIdx.x;
+  if (f8_done(p, b) || (p.bad_a[b] | p.bad_b[b]) != 0) {   // not multiplied, or in FP64 arithmetic anyway
+    if (tid == 0) weak[t] = 0;
+    return;
+  }
+  const int i0 = blockIdx.x / p.ntn * F8_BM, j0 = blockIdx.x % p.ntn * F8_BN;
+  const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
+  const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
+  const int* ea = p.ea + (long long)b * d;
+  const int* eb = p.eb + (long long)b * d;
+  // loads: four entries of A and two of B per thread and slab of K, one slab ahead
+  auto row = [&](int q) { return p.opA ? tid & 127 : (tid >> 4) + 32 * q; };
+  auto ka = [&](int q) { return p.opA ? (tid >> 7) + 4 * q : tid & 15; };
+  const int jb = tid & 63;
+  double2 av[4], bv[2];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + row(q), k = k0 + ka(q);
+      av[q] = make_double2(0.0, 0.0);
+      if (i < d && k < d) av[q] = A[p.opA ? (long long)k * d + i : (long long)i * d + k];
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int k = k0 + (tid >> 6) + 8 * q;
+      bv[q] = make_double2(0.0, 0.0);
+      if (j0 + jb < d && k < d) bv[q] = B[(long long)k * d + j0 + jb];
+    }
+  };
+  load(0);
+  const int Eb = j0 + jb < d ? f8_exponent(eb[j0 + jb]) : 0;
+  int Ea[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) Ea[q] = i0 + row(q) < d ? f8_exponent(ea[i0 + row(q)]) : 0;
+  const int c0 = (tid & 15) * 4, r0 = (tid >> 4) * 4;   // outputs: 4 x 4
+  constexpr float kTiny = 1.1102230246251565e-16f;      // 2^{57 - 110}
+  float m[4][4] = {};
+  bool tiny = false;
+  for (int k0 = 0; k0 < d; k0 += F8_NK) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float v = f8_magnitude(av[q], 57 - Ea[q]);
+      tiny |= v < kTiny && f8_nonzero(av[q]);
+      As[ka(q)][row(q)] = v;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float v = f8_magnitude(bv[q], 57 - Eb);
+      tiny |= v < kTiny && f8_nonzero(bv[q]);
+      Bs[(tid >> 6) + 8 * q][jb] = v;
+    }
+    __syncthreads();
+    if (k0 + F8_NK < d) load(k0 + F8_NK);
+    if (i0 + r0 < d && j0 + c0 < d) {
+#pragma unroll
+      for (int k = 0; k < F8_NK; ++k) {
+        const float4 x = *reinterpret_cast<const float4*>(&As[k][r0]), y = *reinterpret_cast<const float4*>(&Bs[k][c0]);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) m[r][c] = fmaf(xs[r], ys[c], m[r][c]);
+      }
+    }
+    __syncthreads();
+  }
+  const bool any_tiny = __syncthreads_or(tiny);
+  const float per_d = 1.0f / (float)d;
+  bool low = false;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = i0 + r0 + r, j = j0 + c0 + c;
+      if (i >= d || j >= d || m[r][c] >= least || (m[r][c] == 0.f && !any_tiny)) continue;
+      const int k = 114 - f8_exponent(ea[i]) - f8_exponent(eb[j]);
+      float add = i == j ? f8_magnitude(make_double2(p.diag, 0.0), k) : 0.f;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < p.add_n) {
+          const float x = f8_magnitude(reinterpret_cast<const double2*>(p.add_src[q] + b * p.add_stride)[(long long)i * d + j], k);
+          if (x > 0.f) add = fmaf(fabsf((float)p.add_coef[q]), x, add);
+        }
+      low |= !(m[r][c] + add * per_d >= least);
+    }
+  low = __syncthreads_or(low);
+  if (tid == 0) weak[t] = low;
 }
 
-// The marked items in FP64 arithmetic, once a CTA's digit tiles are done: no wait of theirs is
-// open then, however long this takes.  16 x 16 outputs per group of 256 threads (two groups:
-// the epilogue warps), dealt over all groups of the grid; operands through shared memory, sums
-// in the order of cgemm_f64_kernel (the same bits).
-__device__ __noinline__ void f8_pipe_items(const F8Args& p, double2* stage, int et) {
+// The tiles of marked items, and weak ones, in FP64 arithmetic, once a CTA's digit tiles are
+// done: no wait of theirs is open then, however long this takes.  16 x 16 outputs per group of
+// 256 threads (two groups: the epilogue warps), dealt over all groups of the grid; operands
+// through shared memory, sums in the order of cgemm_f64_kernel (the same bits).
+__device__ __noinline__ void f8_pipe_tiles(const F8Args& p, double2* stage, int et) {
   const int g = et >> 8, tx = et & 15, ty = (et >> 4) & 15, d = p.d;
   double2* As = stage + g * (16 * 17 + 16 * 16);   // [k][i], pitch 17
   double2* Bs = As + 16 * 17;                      // [k][j]
-  const int n = (d + 15) / 16, per = n * n;
-  const long long all = 2ll * gridDim.x;
-  long long turn = 2ll * blockIdx.x + g;           // tiles until this group's next one
+  const int per_item = p.ntm * p.ntn;
+  const long long tiles = (long long)per_item * p.batch;
+  const int all = 2 * (int)gridDim.x;
+  int turn = 2 * (int)blockIdx.x + g;              // 16 x 16 outputs until this group's next ones
   auto sync = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); };
-  for (int b = 0; b < p.batch; ++b) {
-    if (!f8_pipe_item(p, b)) continue;
-    const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
-    const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
-    long long u = turn;
-    for (; u < per; u += all) {
-      const int i0 = (int)(u / n) * 16, j0 = (int)(u % n) * 16;
-      double re = 0.0, im = 0.0;
-      for (int k0 = 0; k0 < d; k0 += 16) {
-        double2 v = make_double2(0.0, 0.0), w = v;
-        if (p.opA == 0) {   // A[i0 + ty][k0 + tx]
-          if (i0 + ty < d && k0 + tx < d) v = A[(long long)(i0 + ty) * d + k0 + tx];
-          As[tx * 17 + ty] = v;
-        } else {            // conj(A[k0 + ty][i0 + tx])
-          if (i0 + tx < d && k0 + ty < d) v = A[(long long)(k0 + ty) * d + i0 + tx];
-          As[ty * 17 + tx] = make_double2(v.x, -v.y);
+  for (long long t0 = 0; t0 < tiles; t0 += 32) {
+    const long long tl = t0 + (et & 31);
+    unsigned todo = __ballot_sync(0xffffffffu, tl < tiles && f8_pipe_tile(p, (int)(tl / per_item), tl));
+    for (; todo; todo &= todo - 1) {
+      const long long t = t0 + __ffs(todo) - 1;
+      const int b = (int)(t / per_item), rem = (int)(t % per_item);
+      const double2* A = reinterpret_cast<const double2*>(p.A + b * p.sA);
+      const double2* B = reinterpret_cast<const double2*>(p.B + b * p.sB);
+      constexpr int PER = F8_BM * F8_BN / 256;
+      int u = turn;
+      for (; u < PER; u += all) {
+        const int i0 = rem / p.ntn * F8_BM + u / (F8_BN / 16) * 16, j0 = rem % p.ntn * F8_BN + u % (F8_BN / 16) * 16;
+        if (i0 >= d || j0 >= d) continue;
+        double re = 0.0, im = 0.0;
+        for (int k0 = 0; k0 < d; k0 += 16) {
+          double2 v = make_double2(0.0, 0.0), w = v;
+          if (p.opA == 0) {   // A[i0 + ty][k0 + tx]
+            if (i0 + ty < d && k0 + tx < d) v = A[(long long)(i0 + ty) * d + k0 + tx];
+            As[tx * 17 + ty] = v;
+          } else {            // conj(A[k0 + ty][i0 + tx])
+            if (i0 + tx < d && k0 + ty < d) v = A[(long long)(k0 + ty) * d + i0 + tx];
+            As[ty * 17 + tx] = make_double2(v.x, -v.y);
+          }
+          if (k0 + ty < d && j0 + tx < d) w = B[(long long)(k0 + ty) * d + j0 + tx];
+          Bs[ty * 16 + tx] = w;
+          sync();
+          const int kmax = min(16, d - k0);
+          for (int k = 0; k < kmax; ++k) {
+            const double2 x = As[k * 17 + ty], y = Bs[k * 16 + tx];
+            re = fma(x.x, y.x, re);
+            re = fma(-x.y, y.y, re);
+            im = fma(x.x, y.y, im);
+            im = fma(x.y, y.x, im);
+          }
+          sync();
         }
-        if (k0 + ty < d && j0 + tx < d) w = B[(long long)(k0 + ty) * d + j0 + tx];
-        Bs[ty * 16 + tx] = w;
-        sync();
-        const int kmax = min(16, d - k0);
-        for (int k = 0; k < kmax; ++k) {
-          const double2 x = As[k * 17 + ty], y = Bs[k * 16 + tx];
-          re = fma(x.x, y.x, re);
-          re = fma(-x.y, y.y, re);
-          im = fma(x.x, y.y, im);
-          im = fma(x.y, y.x, im);
+        const int i = i0 + ty, j = j0 + tx;
+        if (i < d && j < d) {
+          const long long off = (long long)i * d + j;
+          for (int m = 0; m < p.add_n; ++m) {
+            const double2 v = reinterpret_cast<const double2*>(p.add_src[m] + b * p.add_stride)[off];
+            re = fma(p.add_coef[m], v.x, re);
+            im = fma(p.add_coef[m], v.y, im);
+          }
+          if (i == j) re += p.diag;
+          reinterpret_cast<double2*>(p.C + b * p.sC)[off] = make_double2(re, im);
         }
-        sync();
       }
-      const int i = i0 + ty, j = j0 + tx;
-      if (i < d && j < d) {
-        const long long off = (long long)i * d + j;
-        for (int m = 0; m < p.add_n; ++m) {
-          const double2 v = reinterpret_cast<const double2*>(p.add_src[m] + b * p.add_stride)[off];
-          re = fma(p.add_coef[m], v.x, re);
-          im = fma(p.add_coef[m], v.y, im);
-        }
-        if (i == j) re += p.diag;
-        reinterpret_cast<double2*>(p.C + b * p.sC)[off] = make_double2(re, im);
-      }
+      turn = u - PER;
     }
-    turn = u - per;
   }
 }
 
@@ -625,7 +752,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   uint64_t* mmadone = accempty + 1;        // closing commit
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mmadone + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* marked_flag = abort_flag + 1;
+  volatile int* pipe_flag = abort_flag + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -637,7 +764,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     mbar_init(accempty, F8_EPI_WARPS);
     mbar_init(mmadone, 1);
     *abort_flag = 0;
-    *marked_flag = 0;
+    *pipe_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -671,7 +798,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int b = (int)(t / per_item);
         int mt, nt;
         f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
-        if (f8_skip(p, b)) continue;
+        if (f8_skip(p, b, t)) continue;
         for (int sweep = 0; sweep < 2 && ok; ++sweep) {
           const int per_step = sweep == 0 ? 4 : 2;
           for (int st = 0; st < steps && ok; ++st) {
@@ -717,7 +844,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       bool ok = !p.stall || f8_wait(mmadone, 0, p.wait_ns, abort_flag);
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         const int b = (int)(t / per_item);
-        if (f8_skip(p, b)) continue;
+        if (f8_skip(p, b, t)) continue;
         for (int sweep = 0; sweep < 2 && ok; ++sweep) {
           const int ns = segments(b, sweep);
           for (int sg = 0; sg < ns && ok; ++sg) {
@@ -789,10 +916,12 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     }
   } else if constexpr (CPLX) {
-    // ---------------- warps 2, 3: is any item marked? ----------------
+    // ---------------- warps 2, 3: does any tile run in FP64 arithmetic? ----------------
     bool any = false;
-    for (int b = threadIdx.x - 64; b < p.batch; b += 64) any |= f8_pipe_item(p, b);
-    if (any) *marked_flag = 1;
+    for (int b = threadIdx.x - 64; b < p.batch; b += 64) any |= (p.bad_a[b] | p.bad_b[b]) != 0 && !f8_done(p, b);
+    if (p.weak)
+      for (long long t = threadIdx.x - 64; t < tiles; t += 64) any |= p.weak[t] != 0;
+    if (any) *pipe_flag = 1;
   }
   } else {
     // ---------------- epilogue (warps 4..19) ----------------
@@ -812,7 +941,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       int mt, nt;
       f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
       const int row0 = mt * F8_BM + q * 32, col0 = nt * 4 * WC + c0;
-      if (f8_skip(p, b)) continue;
+      if (f8_skip(p, b, t)) continue;
       // uniform over the warp; a real tile's columns right of all its rows are not needed
       const bool live = row0 < p.d && col0 < p.d && (CPLX || col0 <= row0 + 31);
       long long acc[F8_VALS];
@@ -972,7 +1101,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         int mt, nt;
         f8_tile<CPLX>(p, (int)(t % per_item), mt, nt);
         const int row = mt * F8_BM + q * 32 + lane;
-        if (f8_skip(p, b) || row >= p.d) continue;
+        if (f8_skip(p, b, t) || row >= p.d) continue;
         const int n0 = nt * 4 * WC + c0;
         for (int c = n0; c < min(p.d, n0 + WC); ++c) {
           if constexpr (CPLX) reinterpret_cast<double2*>(p.C + b * p.sC)[(long long)row * p.d + c] = make_double2(nan, nan);
@@ -990,7 +1119,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
   if constexpr (CPLX)
-    if (warp >= 4 && *marked_flag) f8_pipe_items(p, staging, threadIdx.x - 128);
+    if (warp >= 4 && *pipe_flag) f8_pipe_tiles(p, staging, threadIdx.x - 128);
 }
 
 // ---------------------------------------------------------------------------
@@ -1046,12 +1175,16 @@ int f64d_slice_b(int d, int batch, const double* B, long long sB, void* buf, cud
   return check_launch("f64d_slice_col_kernel");
 }
 
-// scratch of the product (low words between the sweeps): one block per SM
-size_t f64d_scratch_bytes(int sms) { return (size_t)sms * F8_VALS * F8_EPI * sizeof(uint32_t); }
+// scratch of the product: the low words between the sweeps, one block per SM, then a byte per
+// tile (f64d_weak_kernel)
+static size_t f8_low_words_bytes(int sms) { return (size_t)sms * F8_VALS * F8_EPI * sizeof(uint32_t); }
+size_t f64d_scratch_bytes(int sms, int d, int batch) {
+  return f8_low_words_bytes(sms) + (size_t)ceil_div(d, F8_BM) * ceil_div(d, F8_BN) * batch;
+}
 
 int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const void* abuf, const double* B,
               long long sB, const void* bbuf, double* C, long long sC, const AddTerms& add, void* scratch, int sms,
-              int* status, cudaStream_t s, const SplitCtl& ctl) {
+              bool entrywise, int* status, cudaStream_t s, const SplitCtl& ctl) {
   if (batch <= 0) return MG_OK;
   if (batch > 65535) return MG_EUNSUPPORTED;
   if (add.scale != 1.0) return MG_EINVAL;
@@ -1090,6 +1223,13 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   p.sq_step = ctl.sq_step;
   p.stall = ctl.stall;
   p.wait_ns = std::min<unsigned long long>(ctl.wait_ns, 4000000000ull);
+  if (entrywise) {
+    unsigned char* weak = static_cast<unsigned char*>(scratch) + f8_low_words_bytes(sms);
+    const float least = ldexpf(1.0f, 114 - 8) / sqrtf((float)d);
+    f64d_weak_kernel<<<dim3(p.ntm * p.ntn, batch), F8_WEAK_THREADS, 0, s>>>(p, least, weak);
+    MG_TRY(check_launch("f64d_weak_kernel"));
+    p.weak = weak;
+  }
   // one CTA per tile up to one per SM, and no fewer than marked items' 16 x 16 tiles would fill
   const long long tiles = (long long)p.ntn * p.ntm * batch, sub = ceil_div(d, 16);
   const int grid = (int)std::min<long long>(std::max(tiles, (sub * sub * batch + 1) / 2), sms);
