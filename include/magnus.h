@@ -63,7 +63,8 @@ extern "C" {
  *   base-256 digits per operand (63 bits below every row's or column's largest entry, exact
  *   level sums, one rounding per entry); their error is below FP64 arithmetic's, relative to
  *   the largest entries of A's row and B's column: in a propagator, an amplitude 2^-k below
- *   the largest of its row holds about 60 - k bits (FP64 arithmetic 53 whatever k).  Where the
+ *   the largest of its row holds about 60 - k bits (FP64 arithmetic 53 whatever k; a context
+ *   can ask for that throughout, mg_ctx_set_fp64_entrywise).  Where the
  *   operands are the caller's -- mg_expm, mg_propagate, the running product of an evolution
  *   resumed from `in` -- every entry holds FP64 arithmetic's bound, about
  *   d 2^-53 sum_k |a_ik| |b_kj|: 128 x 64 blocks with weaker entries than the digits hold so
@@ -607,6 +608,12 @@ int mg_ctx_set_cta_pairs(mg_ctx* ctx, int on);
  * the d (d + 1) / 2 entries on and below the diagonal of a symmetric result.  MG_EINVAL
  * outside 0..3. */
 int mg_ctx_set_structure(mg_ctx* ctx, int on);
+/* MG_PREC_FP64 entry by entry: on != 0 runs every FP64 product of the context's calls in native
+ * FP64 arithmetic, also those that digits would give (evolutions, batches, servers; the
+ * products of re-orthonormalisation and of the report in either precision), so that weak
+ * amplitudes keep 53 bits of their own.  One product of d = 729: 2.6 ms instead of 0.1.
+ * 0 (the default) as described at MG_PREC_FP64. */
+int mg_ctx_set_fp64_entrywise(mg_ctx* ctx, int on);
 int mg_ctx_gemm_stats(mg_ctx* ctx, int64_t* launches, double* ms, double* flops, int reset);
 
 const char* mg_strerror(int code);

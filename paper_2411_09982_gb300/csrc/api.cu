@@ -125,6 +125,7 @@ struct mg_ctx {
   unsigned long long wait_ns = 4000000000ull;
   int stall_test = 0;
   int sms = 1;                // multiprocessors of the device
+  int fp64_native = 0;        // no FP64 product from digits (mg_ctx_set_fp64_entrywise)
   // algorithmic work of predicated squaring launches, added on the device (timing on)
   double* dev_flops = nullptr;
   std::string tune_cache;   // tuning cache consulted by servers for MG_PREC_AUTO jobs
@@ -391,8 +392,10 @@ struct Engine {
   // bound entry by entry (products from digits check for it)
   bool entrywise = false;
   // FP64 products from integer digits on the tensor cores (gemm_f64_digits.cu)
-  bool digits64(int batch) const { return prec == MG_PREC_FP64 && !fp64_pipe && f64_digits_pay(d, batch); }
-  bool digits_dim() const { return prec == MG_PREC_FP64 && !fp64_pipe && d >= kF64DigitsMinDim; }   // some batch may
+  bool digits64(int batch) const { return digits_dim() && f64_digits_pay(d, batch); }
+  bool digits_dim() const {   // some batch may
+    return prec == MG_PREC_FP64 && !fp64_pipe && !ctx->fp64_native && d >= kF64DigitsMinDim;
+  }
   bool allow18() const { return prec == MG_PREC_SPLIT && taylor_mode != MG_TAYLOR_PS; }
   SplitCtl ctl() const {
     SplitCtl c;
@@ -1454,6 +1457,12 @@ int mg_ctx_set_digit_pairs(mg_ctx* ctx, int on) {
 int mg_ctx_set_structure(mg_ctx* ctx, int on) {
   if (!ctx || on < 0 || on > 3) return MG_EINVAL;
   ctx->structure = on;
+  return MG_OK;
+}
+
+int mg_ctx_set_fp64_entrywise(mg_ctx* ctx, int on) {
+  if (!ctx) return MG_EINVAL;
+  ctx->fp64_native = on != 0;
   return MG_OK;
 }
 

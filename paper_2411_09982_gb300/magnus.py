@@ -121,6 +121,7 @@ SIGNATURES = {
     "mg_ctx_set_digit_pairs": (_I, [_P, _I]),
     "mg_ctx_set_cta_pairs": (_I, [_P, _I]),
     "mg_ctx_set_structure": (_I, [_P, _I]),
+    "mg_ctx_set_fp64_entrywise": (_I, [_P, _I]),
     "mg_ctx_gemm_stats": (_I, [_P, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(_D), ctypes.POINTER(_D), _I]),
     "mg_cgemm_split_static": (_I, [_I, _P, _I, _I, _P, _P, _P, _I]),
     "mg_tune_select": (_I, [_I, ctypes.POINTER(mg_tune_entry), _D, _D, ctypes.POINTER(_I)]),
@@ -226,6 +227,10 @@ class Context:
         bit 1 the tiles above the diagonal of symmetric results; True = 3 (default), False = 0."""
         mode = 3 if mode is True else (0 if mode is False else int(mode))
         _check(load().mg_ctx_set_structure(self.h, mode), "mg_ctx_set_structure")
+
+    def set_fp64_entrywise(self, on=True):
+        """Every FP64 product in native FP64 arithmetic: weak amplitudes keep all their bits."""
+        _check(load().mg_ctx_set_fp64_entrywise(self.h, 1 if on else 0), "mg_ctx_set_fp64_entrywise")
 
     def set_wait_limit(self, seconds=4.0, stall_test=False):
         _check(load().mg_ctx_set_wait_limit(self.h, float(seconds), 1 if stall_test else 0), "mg_ctx_set_wait_limit")

@@ -1,6 +1,6 @@
 """Weak entries in MG_PREC_FP64: products of arbitrary operands (mg_propagate, mg_expm, a resumed
 run's running product) hold FP64's error entry by entry, |error| <= c u |A| |B|, whatever the
-range of a row's entries."""
+range of a row's entries; and so does every product under Context.set_fp64_entrywise(True)."""
 import numpy as np
 import pytest
 
@@ -109,6 +109,37 @@ def test_resumed_running_product(call):
             assert M.mg_evolve_batch(ctx, [plan], [M.MG_OUT_PROPAGATOR], [cuda(inp)], [out]) == [0]
         got = out.cpu().numpy()
         assert np.abs(got[0, 1:] - got[0, 0] * inp[0, 1:]).max() <= 8 * 2.0 ** -53 * np.abs(inp[0, 1:]).max()
+        plan.close()
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("real", [True, False])
+@pytest.mark.parametrize("d", [20, 40, 130, 209])
+def test_every_product_when_asked_for(d, real):
+    """set_fp64_entrywise: evolutions keep weak amplitudes (exponentials, tree and running products)."""
+    rng = np.random.default_rng(d)
+    e = 2.0 ** -50
+    N = 2 * enough(d) if d > 32 else 8
+    ctx = M.Context(0)
+    try:
+        A, ref = weakly_coupled(rng, d, e, real)
+        ctx.set_fp64_entrywise(True)
+        plan = M.Plan(ctx, cuda(A), None, M.MG_PREC_FP64)
+        plan.set_controls(N, 1, 0.0, 1.0 / N, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
+        for output in (M.MG_OUT_PROPAGATOR, M.MG_OUT_STATE):
+            if output == M.MG_OUT_PROPAGATOR:
+                out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+                plan.evolve(output, None, out)
+                got, want = out.cpu().numpy()[:d // 2, d // 2:], ref
+            else:
+                psi = np.zeros(d, dtype=np.complex128)
+                psi[d - 1] = 1.0
+                out = torch.empty(d, dtype=torch.complex128, device="cuda")
+                plan.evolve(output, cuda(psi), out)
+                got, want = out.cpu().numpy()[:d // 2], ref[:, -1]
+            # N intervals of ~10 products of d-term sums
+            assert np.abs(got - want).max() <= 2.0 ** -53 * 200 * d * np.abs(ref).max()
         plan.close()
     finally:
         ctx.close()
