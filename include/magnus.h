@@ -598,7 +598,8 @@ int mg_ctx_set_cta_pairs(mg_ctx* ctx, int on);
  *          on and below the diagonal, entry (i, j) with j > i read as (j, i); each U_n is
  *          written in full, exactly symmetric, the same on either tiling, and differs from
  *          the full products' by their own rounding asymmetry.  The tree product of the
- *          U_n is general.
+ *          U_n is general.  In MG_PREC_FP64 (where bit 0 has no effect) it forms each U_n
+ *          as cos A - i sin A from real symmetric products of d^2 (d + 1) flops each.
  * 3 (the default) sets both, 0 issues every product in full.  Applies to mg_evolve,
  * mg_evolve_batch (a batch only when all of its plans qualify) and the chunk steps of a
  * server (mg_submit checks each job's operators; a step only when all of its jobs

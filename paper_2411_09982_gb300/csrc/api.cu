@@ -537,8 +537,10 @@ struct Engine {
     return MG_OK;
   }
   int timing_begin(int* idx) { return timing_mark(ctx, idx); }
-  // FP64 exponentials of real symmetric exponents from digits
-  bool real64(int batch) const { return digits64(batch) && x_sym; }
+  // FP64 exponentials of real symmetric exponents as cosine and sine: symmetric products, so
+  // bit 1 of the structure option
+  bool x_real() const { return x_sym && (ctx->structure & 2); }
+  bool real64(int batch) const { return digits64(batch) && x_real(); }
   // real products on the lower triangle that degree m and sq squarings take
   static int real_products(int m, int sq) {
     const int kc = m / 2, ks = (m - 1) / 2, p = (kc + 1) / 2;
@@ -578,13 +580,13 @@ struct Engine {
     products += (long long)batch * (per_poly + sq);
     int e0 = -1, e1 = -1;
     if (ctx->timing) MG_TRY(timing_begin(&e0));
-    MG_TRY(launch_expm_small(batch, d, W, tau, m, p, sq, sq_dev, x_sym ? 1 : 0, U, ctx->stream));
+    MG_TRY(launch_expm_small(batch, d, W, tau, m, p, sq, sq_dev, x_real() ? 1 : 0, U, ctx->stream));
     if (ctx->timing) {
       MG_TRY(timing_begin(&e1));
       ctx->ev_pending.emplace_back(e0, e1);
       ctx->t_launches += 1;
       // the flops issued: real products of the lower triangle, or complex ones
-      const double work = x_sym ? (double)d * d * (d + 1) * real_products(m, sq_dev ? 0 : sq)
+      const double work = x_real() ? (double)d * d * (d + 1) * real_products(m, sq_dev ? 0 : sq)
                                 : 8.0 * d * d * d * (per_poly + (sq_dev ? 0 : sq));
       ctx->t_flops += work * batch;
     }

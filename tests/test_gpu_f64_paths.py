@@ -28,8 +28,8 @@ def exact(A):
     return (V * np.exp(-1j * lam)) @ V.conj().T
 
 
-def one_plan(ctx, A, N):
-    plan = M.Plan(ctx, cuda(A), None, M.MG_PREC_FP64)
+def one_plan(ctx, A, N, prec=M.MG_PREC_FP64):
+    plan = M.Plan(ctx, cuda(A), None, prec)
     plan.set_controls(N, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
     return plan
 
@@ -75,5 +75,33 @@ def test_batch_of_complex_exponents_with_uneven_squarings():
             norm = np.abs(A - np.trace(A) / len(A) * np.eye(len(A))).sum(0).max()
             # N intervals of ~20 products of d-term sums, doubled by every squaring
             assert np.abs(o.cpu().numpy() - exact(N * A)).max() <= N * 2.0 ** -53 * 20 * 80 * (1 + 4 * norm)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("d", [20, 40, 130])
+def test_structure_option_issues_products_in_full(d):
+    """Structure 0: complex products of 8 d^3 each; 3: the real symmetric form, fewer; the same U."""
+    rng = np.random.default_rng(d)
+    N = enough(d) if d > 32 else 4
+    A = hermitian(rng, d, 3.0, True)
+    ctx = M.Context(0)
+    try:
+        outs, flops = [], []
+        for mode in (0, 1, 2, 3):
+            ctx.set_structure(mode)
+            ctx.enable_gemm_timing(True)
+            ctx.gemm_stats(reset=True)
+            plan = one_plan(ctx, A, N)
+            psi = np.eye(d)[0].astype(np.complex128)
+            traj = torch.empty((N + 1, d), dtype=torch.complex128, device="cuda")   # a trajectory takes no products beside the exponentials'
+            rep = plan.evolve(M.MG_OUT_TRAJECTORY, cuda(psi), traj)
+            flops.append(ctx.gemm_stats()["flops"] / (8.0 * d ** 3 * rep["matrix_products"]))
+            outs.append(traj[1].cpu().numpy())
+            plan.close()
+        assert abs(flops[0] - 1) <= 1e-12 and abs(flops[1] - 1) <= 1e-12 and flops[2] < 0.6 and flops[3] == flops[2]
+        for o in outs:
+            assert np.abs(o - exact(A)[:, 0]).max() <= 2.0 ** -53 * 20 * d * 13
+        assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[2], outs[3])
     finally:
         ctx.close()
