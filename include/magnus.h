@@ -510,7 +510,10 @@ int mg_cgemm_split_static(int device, void* stream, int batch, int d, const doub
  * product launch on its stream; mg_ctx_gemm_stats synchronises the stream and
  * returns the number of launches, their summed device time (ms) and their
  * summed algorithmic work (8 d^3 real flops per complex d x d product, the
- * 4-real-multiplication form), then optionally resets the counters.  The
+ * 4-real-multiplication form; less where the operands' structure is used, see
+ * mg_ctx_set_structure), then optionally resets the counters.  In MG_PREC_FP64
+ * a chunk's exponentials in the cosine and sine form, or of d <= 32, count as
+ * one launch, with the time of their elementwise steps.  The
  * action kernel of MG_FLAG_STATE_ACTION counts as one launch with 8 flops per
  * stored operator nonzero per operator application. */
 int mg_ctx_enable_gemm_timing(mg_ctx* ctx, int enable);

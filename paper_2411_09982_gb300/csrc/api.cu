@@ -571,6 +571,12 @@ struct Engine {
     }
     return MG_OK;
   }
+  // algorithmic flops of one squaring of a batch's exponential, by the form it takes
+  double squaring_flops(int batch) const {
+    const double cube = (double)d * d * d, lower = (double)d * d * (d + 1);
+    if (prec == MG_PREC_SPLIT) return x_sym && (ctx->structure & 2) ? 4.0 * lower : 8.0 * cube;
+    return real64(batch) || (small64() && x_real()) ? 2.0 * lower : 8.0 * cube;
+  }
   // FP64 exponentials in one launch (expm_small.cu)
   bool small64() const { return prec == MG_PREC_FP64 && d <= expm_small_max_dim(); }
   // per_poly products of the polynomial and sq squarings (sq_dev: per item, at most sq) are
@@ -2598,7 +2604,7 @@ int issue_chunk(mg_ctx* ctx, Engine& eng, GroupProgram& G, ChunkPlan& ch) {
   MG_TRY(launch_fail_segments((int)ch.segs.size(), fill, md, G.itab + ch.seg_tab, G.itab + ch.seg_of_item, nrm, tau,
                               G.job_fail, G.seg_bad, W, s));
   MG_TRY(launch_squarings(fill, nrm, G.tc.theta, G.S, 0, G.sq, G.overflow, ctx->timing ? ctx->dev_flops : nullptr,
-                          8.0 * (double)dp * dp * dp, s));
+                          eng.squaring_flops(fill), s));
   MG_TRY(expm_chunk_dev(ctx, eng, fill, W, tau, G.sq, G.tc, G.S, Ub, eng.df()));
   PhaseRange pr("propagate");
   // propagator jobs: tree product of the segment, folded into the running product

@@ -105,3 +105,30 @@ def test_structure_option_issues_products_in_full(d):
         assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[2], outs[3])
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "split"])
+@pytest.mark.parametrize("real", [True, False])
+@pytest.mark.parametrize("d", [32, 48])   # a batch pads d to a multiple of 16
+def test_batch_counts_the_work_that_an_evolution_counts(d, real, prec):
+    """The squarings of a batch are counted on the device, those of mg_evolve on the host."""
+    rng = np.random.default_rng(d)
+    N = 2 * enough(d) if d > 32 else 8
+    A = hermitian(rng, d, 5.0, real)
+    ctx = M.Context(0)
+    try:
+        ctx.enable_gemm_timing(True)
+        plan = one_plan(ctx, A, N, M.MG_PREC_FP64 if prec == "fp64" else M.MG_PREC_SPLIT)
+        flops = []
+        for batch in (False, True):
+            ctx.gemm_stats(reset=True)
+            out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+            if batch:
+                assert M.mg_evolve_batch(ctx, [plan], [M.MG_OUT_PROPAGATOR], [None], [out]) == [0]
+            else:
+                plan.evolve(M.MG_OUT_PROPAGATOR, None, out, report=False)
+            flops.append(ctx.gemm_stats()["flops"])
+        assert abs(flops[1] / flops[0] - 1) <= 1e-12
+        plan.close()
+    finally:
+        ctx.close()
