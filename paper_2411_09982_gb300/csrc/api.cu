@@ -881,25 +881,35 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
 }
 
 // C = opA(A) B in FP64 (report and re-orthonormalisation products): from digits where the
-// engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`.  Entry
-// by entry only where the engine's products are FP64 ones (split states carry larger errors,
-// and the report takes the largest entry of its product).
+// engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`, as many
+// items at a time as those hold (split precision with few slices reserves less than FP64
+// digits take).  Entry by entry only where the engine's products are FP64 ones (split states
+// carry larger errors, and the report takes the largest entry of its product).
 int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const double* B, double* C) {
   const long long md = mat_doubles(eng.d);
   AddTerms none;
   Engine e{ctx, eng.d, MG_PREC_FP64, 0};
-  if (!e.digits64(batch)) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
+  int nb = batch;
+  if (e.digits_dim() && eng.abuf && eng.bbuf[0])
+    nb = (int)std::min<size_t>(nb, std::max<size_t>(1, std::min(ctx->slot_size[WS_ABUF] / f64d_a_bytes(e.d, 1),
+                                                                ctx->slot_size[WS_BBUF0] / f64d_b_bytes(e.d, 1))));
+  if (!e.digits64(nb)) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
   void *ab, *bb, *sums;
-  MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, batch), &ab));
-  MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(e.d, batch), &bb));
-  MG_TRY(ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms, e.d, batch), &sums));
-  if (eng.abuf) eng.abuf = ab;   // the slots may have grown
+  MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, nb), &ab));
+  MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(e.d, nb), &bb));
+  MG_TRY(ws_get(ctx, WS_F64_SUMS, f64d_scratch_bytes(ctx->sms, e.d, nb), &sums));
+  if (eng.abuf) eng.abuf = ab;   // the slots may have grown (to one item)
   if (eng.bbuf[0]) eng.bbuf[0] = bb;
   const SplitCtl c = e.ctl();
-  MG_TRY(f64d_slice_a(e.d, batch, A, md, opA, ab, ctx->stream, c));
-  MG_TRY(f64d_slice_b(e.d, batch, B, md, bb, ctx->stream, c));
-  return f64d_gemm(e.d, batch, opA, A, md, ab, B, md, bb, C, md, none, sums, ctx->sms, eng.entrywise && !eng.df(),
-                  ctx->status, ctx->stream, c);
+  for (int b0 = 0; b0 < batch; b0 += nb) {
+    const int n = std::min(nb, batch - b0);
+    const double *Ai = A + b0 * md, *Bi = B + b0 * md;
+    MG_TRY(f64d_slice_a(e.d, n, Ai, md, opA, ab, ctx->stream, c));
+    MG_TRY(f64d_slice_b(e.d, n, Bi, md, bb, ctx->stream, c));
+    MG_TRY(f64d_gemm(e.d, n, opA, Ai, md, ab, Bi, md, bb, C + b0 * md, md, none, sums, ctx->sms,
+                     eng.entrywise && !eng.df(), ctx->status, ctx->stream, c));
+  }
+  return MG_OK;
 }
 
 // One Newton-Schulz polar step in FP64 on a batch: Z <- Z (3I - Z^dag Z)/2.
@@ -966,21 +976,33 @@ int tree_product(mg_ctx* ctx, Engine& eng, int n, const double* U, double** out,
 
 // Device bytes one interval of a chunk needs: Hbar/X, X^2, X^3, Y, two Horner
 // buffers, the chunk's U_n, tree and re-orthonormalisation scratch (about
-// 9 matrices), plus the BF16 digits of one A and two B operands.
-size_t per_interval_bytes(int d, int prec, int L) {
+// 9 matrices), plus the digits of one A and two B operands.
+size_t per_interval_bytes(int d, int prec, int L, bool digits) {
   size_t md = (size_t)mat_doubles(d) * sizeof(double);
   size_t b = 10 * md;   // (one more for the gathered pairs of a segmented tree)
   if (prec == MG_PREC_SPLIT) b += split_a_bytes(d, L, 1) + 2 * split_b_bytes(d, L, 1);
-  else if (d >= kF64DigitsMinDim) b += f64d_a_bytes(d, 1) + 2 * f64d_b_bytes(d, 1);
+  else if (digits) b += f64d_a_bytes(d, 1) + 2 * f64d_b_bytes(d, 1);
   return b;
 }
 
-int chunk_size(mg_ctx* ctx, int d, int prec, int L, int N, int align) {
-  const size_t per = per_interval_bytes(d, prec, L);
-  long long c = (long long)(ctx->ws_limit / per);
+// may_digits: the call's FP64 products may run from digits
+int chunk_size(mg_ctx* ctx, int d, int prec, int L, int N, int align, bool may_digits = true) {
+  auto fit = [&](size_t bytes, size_t per) { return std::min<long long>((long long)(bytes / per), std::min(N, 4096)); };
+  const bool digits = prec == MG_PREC_FP64 && may_digits && !ctx->fp64_native;
+  long long c = fit(ctx->ws_limit, per_interval_bytes(d, prec, L, false));
+  if (digits && f64_digits_pay(d, (int)std::max(c, 1ll))) {
+    // FP64 with room for digits, or the most intervals that do without
+    const long long dp = (d + 15) / 16 * 16, without = 7999999 / (dp * dp * dp);
+    c = std::max(fit(ctx->ws_limit, per_interval_bytes(d, prec, L, true)), std::min(c, without));
+  }
+  if (prec == MG_PREC_SPLIT && may_digits && !ctx->fp64_native && f64_digits_pay(d, 1)) {
+    // FP64 digits of one item (report, re-orthonormalisation) beyond what the chunk's slots hold
+    auto beyond = [&](long long n, size_t f64, size_t split) { return f64 > n * split ? f64 - n * split : 0; };
+    const size_t fa = f64d_a_bytes(d, 1), fb = f64d_b_bytes(d, 1), sa = split_a_bytes(d, L, 1), sb = split_b_bytes(d, L, 1);
+    const size_t more = beyond(c, fa, sa) + beyond(c, fb, sb);
+    if (more > 0 && more < ctx->ws_limit) c = std::min(c, fit(ctx->ws_limit - more, per_interval_bytes(d, prec, L, false)));
+  }
   if (c < 1) c = 1;
-  if (c > 4096) c = 4096;
-  if (c > N) c = N;
   if (align > 1 && c > align) c = (c / align) * align;
   return (int)c;
 }
@@ -1746,7 +1768,7 @@ int mg_cgemm(mg_ctx* ctx, int batch, int d, const double* A, const double* B, do
   // digits' to the largest entries of A's row and B's column
   eng.fp64_pipe = true;
   const long long md = mat_doubles(d);
-  const int chunk = std::min(chunk_size(ctx, d, precision, slices, batch, 1), 65535);
+  const int chunk = std::min(chunk_size(ctx, d, precision, slices, batch, 1, false), 65535);
   for (int b0 = 0; b0 < batch; b0 += chunk) {
     int nb = std::min(chunk, batch - b0);
     MG_TRY(eng.reserve(nb));

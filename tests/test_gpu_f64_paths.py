@@ -132,3 +132,50 @@ def test_batch_counts_the_work_that_an_evolution_counts(d, real, prec):
         plan.close()
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("case", ["reorth", "report"])
+def test_workspace_stays_within_its_limit(case):
+    """Split precision with two slices: the FP64 digits of re-orthonormalisation and of the
+    report's product are four times its own operands'.  The context's pool (device memory taken
+    during the call) holds no more than the limit and 2 MiB of rounding per buffer."""
+    rng = np.random.default_rng(0)
+    d, N = 1024, 24 if case == "reorth" else 2
+    md = 16 * d * d
+    limit = 260 * md if case == "reorth" else 25 * md
+    A = hermitian(rng, d, 1.0, False)
+
+    def taken(N, reorth, limit):
+        ctx = M.Context(0, workspace_limit=limit)
+        plan = M.Plan(ctx, cuda(A), None, M.MG_PREC_SPLIT, 2)
+        plan.set_controls(N, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
+        out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        plan.evolve(M.MG_OUT_PROPAGATOR, None, out, reorth)
+        used = before - torch.cuda.mem_get_info()[0]
+        plan.close()
+        ctx.close()
+        return used
+
+    taken(2, 2, limit)   # loads every kernel of the path
+    assert taken(N, 2 if case == "reorth" else 0, limit) <= limit + 20 * (2 << 20)
+
+
+def test_fp64_chunks_without_digits_are_not_cut_for_them():
+    """64 products of d = 40 run on the FP64 pipe: a limit that fits 64 intervals without digits
+    runs them in one chunk, as any larger one."""
+    rng = np.random.default_rng(0)
+    d, N = 40, 64
+    A = hermitian(rng, d, 1.0, False)
+    launches = []
+    for limit in (1 << 30, N * 10 * 16 * d * d):
+        ctx = M.Context(0, workspace_limit=limit)
+        plan = one_plan(ctx, A, N)
+        out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+        before = M.mg_kernel_launch_count()
+        plan.evolve(M.MG_OUT_PROPAGATOR, None, out)
+        launches.append(M.mg_kernel_launch_count() - before)
+        plan.close()
+        ctx.close()
+    assert launches[0] == launches[1]
