@@ -336,7 +336,7 @@ f64d_slice_col_kernel(int d, int Kp, const double2* __restrict__ B, long long sB
 // warp per row: entry k is X[k] + sz Z[k] (Z null: X[k]), or with CW the real part of a complex
 // matrix W times 2^{-sq} (an exact change of the row's exponent).  grid (ceil(d / 8), batch).
 // Entries are bounded above (the exponential scales them to norm about 1) and finite, so no
-// row is marked; the product takes scales down to the smallest subnormal (f8_value_any).
+// row is marked; the product takes scales down to the smallest subnormal (f8_value).
 template <bool CW>
 __global__ void __launch_bounds__(256)
 f64r_slice_kernel(int d, int Kh, const double* __restrict__ X, const double* __restrict__ Z, double sz, long long sX,
@@ -653,7 +653,9 @@ __device__ __forceinline__ bool f8_wait(uint64_t* bar, uint32_t parity, unsigned
   return true;
 }
 
-// (t 2^32 + w) 2^k rounded to FP64, |t| < 2^63; k keeps the result a normal number.
+// (t 2^32 + w) 2^k rounded to FP64, |t| < 2^63; k keeps the result below 2^1024, and with
+// TINY = false above FP64's smallest normal number (otherwise what lies below that becomes 0).
+template <bool TINY>
 __device__ __forceinline__ double f8_value(long long t, uint32_t w, int k) {
   const uint32_t neg = (uint32_t)((unsigned long long)t >> 63);
   const unsigned long long s = 0ull - neg;
@@ -674,24 +676,17 @@ __device__ __forceinline__ double f8_value(long long t, uint32_t w, int k) {
   // 53 bits and the rounding bit; a carry runs into the exponent as it should
   const unsigned long long m = ((unsigned long long)m1 << 32 | m0) >> 11;
   const unsigned long long bits = ((unsigned long long)(uint32_t)(e - lz) << 52) + m + ((m0 >> 10) & 1u);
-  return t1 == 0u ? 0.0 : __longlong_as_double((long long)(bits | (unsigned long long)neg << 63));
+  return t1 == 0u || (TINY && e <= lz) ? 0.0 : __longlong_as_double((long long)(bits | (unsigned long long)neg << 63));
 }
 
 // The same on the FP64 pipe, |t| < 2^51.  A warp's FP64 instruction takes about 68 cycles of
 // its quarter of the SM, the integer form some 50 dependent instructions: the epilogues send
 // every fourth value here, which is where the two balance.
 __device__ __forceinline__ double f8_value_fp64(long long t, uint32_t w, int k) {
-  const double h = __longlong_as_double(t + 0x4338000000000000ll) - 6755399441055744.0;   // (1.5 2^52 + t) - 1.5 2^52
-  const double l = __hiloint2double(0x43300000, (int)w) - 4503599627370496.0;             // (2^52 + w) - 2^52
-  return fma(h, 4294967296.0, l) * __hiloint2double((k + 1023) << 20, 0);
-}
-
-// Either of the two for any k: real rows may be scaled down to the smallest subnormal.
-template <bool PIPE>
-__device__ __forceinline__ double f8_value_any(long long t, uint32_t w, int k) {
-  const bool tiny = k < -1000;
-  const double x = PIPE ? f8_value_fp64(t, w, tiny ? -60 : k) : f8_value(t, w, tiny ? -60 : k);
-  return tiny ? scalbn(x, k + 60) : x;
+  // t 2^-64 and w 2^-96, exact: (1.5 2^52 + t) 2^-64 - 1.5 2^-12, (2^52 + w) 2^-96 - 2^-44
+  const double h = __longlong_as_double(t + 0x3F38000000000000ll) - 0.0003662109375;
+  const double l = __hiloint2double(0x3D300000, (int)w) - 5.684341886080802e-14;
+  return (h + l) * __hiloint2double(max(k + 96 + 1023, 0) << 20, 0);   // 2^{k + 96}; 0 from k = -1119 down
 }
 
 // Drain of one accumulator set (levels l0 .. l0 + 3) into the thread's sums, in units of
@@ -1008,7 +1003,7 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int v = 0; v < 8; ++v) {
               const int col = col0 + c + v;
               const int k = Ea + (col < p.d ? f8_exponent(ebp[col]) : 0) - 68 + p.scale2;
-              double x = v % 4 == 3 ? f8_value_any<true>(acc[c + v], w[v], k) : f8_value_any<false>(acc[c + v], w[v], k);
+              double x = v % 4 == 3 ? f8_value_fp64(acc[c + v], w[v], k) : f8_value<true>(acc[c + v], w[v], k);
               if (row < p.d && col <= row) {
                 const long long off = (long long)col * p.d + row;
 #pragma unroll
@@ -1060,8 +1055,8 @@ f64d_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             // the value is (sum 2^32 + low word) 2^{Ea + Eb - 68}, in units of 2^-56; every
             // fourth goes over the FP64 pipe
             const int k = Ea + __shfl_sync(0xffffffffu, Eb, c + v) - 68;
-            const double re = f8_value(acc[c + v], wre[v], k);
-            const double im = v & 1 ? f8_value_fp64(acc[WC + c + v], wim[v], k) : f8_value(acc[WC + c + v], wim[v], k);
+            const double re = f8_value<false>(acc[c + v], wre[v], k);
+            const double im = v & 1 ? f8_value_fp64(acc[WC + c + v], wim[v], k) : f8_value<false>(acc[WC + c + v], wim[v], k);
             stg[lane * 4 + (v ^ ((lane >> 1) & 3))] = make_double2(re, im);
           }
           __syncwarp();
