@@ -46,6 +46,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <tuple>
 
 namespace mg {
 
@@ -580,23 +581,63 @@ action_rows_kernel(ActionJob* __restrict__ jobs, int dmax) {
   if (C > 1) cl.sync();   // no CTA leaves while another may still address its shared memory
 }
 
-template <int R>
-static int launch_action_rows(int njobs, ActionJob* jobs_dev, int dmax, int C, cudaStream_t s) {
-  auto kern = action_rows_kernel<R>;
+using ActionRowsKernel = void (*)(ActionJob*, int);
+static ActionRowsKernel action_rows_form(int row_regs) {
+  return row_regs == 8 ? action_rows_kernel<8> : row_regs == 16 ? action_rows_kernel<16> : action_rows_kernel<24>;
+}
+static int action_rows_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, ActionRowsKernel kern, int njobs,
+                              int dmax, int C, cudaStream_t s) {
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(kern), ACTION_SMEM_LIMIT));
   MG_TRY(ensure_func_attr(reinterpret_cast<const void*>(kern), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(njobs * C, 1, 1);
-  cfg.blockDim = dim3((2 * ((dmax + C - 1) / C) + 31) / 32 * 32, 1, 1);
-  cfg.dynamicSmemBytes = 4 * sizeof(double) * (size_t)dmax;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3(njobs * C, 1, 1);
+  cfg->blockDim = dim3((2 * ((dmax + C - 1) / C) + 31) / 32 * 32, 1, 1);
+  cfg->dynamicSmemBytes = 4 * sizeof(double) * (size_t)dmax;
+  cfg->stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+  return MG_OK;
+}
+
+// Largest cluster size <= want (a power of two) of the real-row kernel that the device can
+// co-schedule with at most 256 rows per CTA, or 1; answers are cached per form and size.
+int action_rows_cluster_size(int want, int dmax, int row_regs) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int>, bool> fits;
+  const ActionRowsKernel kern = action_rows_form(row_regs);
+  for (int C = want; C >= 2; C >>= 1) {
+    if ((dmax + C - 1) / C > 256) return 1;
+    const std::tuple<int, int, int> key{row_regs, C, dmax};
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      auto it = fits.find(key);
+      if (it != fits.end()) {
+        if (it->second) return C;
+        continue;
+      }
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    int active = 0;
+    const bool ok = action_rows_config(&cfg, attr, kern, 1, dmax, C, nullptr) == MG_OK &&
+                    cudaOccupancyMaxActiveClusters(&active, kern, &cfg) == cudaSuccess && active >= 1;
+    if (!ok) cudaGetLastError();
+    std::lock_guard<std::mutex> lock(mu);
+    fits[key] = ok;
+    if (ok) return C;
+  }
+  return 1;
+}
+
+static int launch_action_rows(int row_regs, int njobs, ActionJob* jobs_dev, int dmax, int C, cudaStream_t s) {
+  const ActionRowsKernel kern = action_rows_form(row_regs);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  MG_TRY(action_rows_config(&cfg, attr, kern, njobs, dmax, C, s));
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, jobs_dev, dmax);
   if (e != cudaSuccess) {
     set_last_cuda_error(e, "cudaLaunchKernelEx(action_rows_kernel)", __FILE__, __LINE__);
@@ -699,9 +740,7 @@ int launch_action_chain(int njobs, ActionJob* jobs_dev, int dmax, int nmax, int 
     action_bounds_kernel<<<grid, 256, 0, s>>>(jobs_dev);
     MG_TRY(check_launch("action_bounds_kernel"));
   }
-  if (row_regs == 8) return launch_action_rows<8>(njobs, jobs_dev, dmax, cluster, s);
-  if (row_regs == 16) return launch_action_rows<16>(njobs, jobs_dev, dmax, cluster, s);
-  if (row_regs == 24) return launch_action_rows<24>(njobs, jobs_dev, dmax, cluster, s);
+  if (row_regs) return launch_action_rows(row_regs, njobs, jobs_dev, dmax, cluster, s);
   if (cluster > 1) return launch_action_cluster(njobs, jobs_dev, dmax, cluster, nnz_cap, s);
   const size_t smem = action_smem_bytes(dmax, nnz_cap);
   MG_TRY(action_attrs());

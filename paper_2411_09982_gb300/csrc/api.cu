@@ -1175,9 +1175,10 @@ bool shape_action_rows(const std::vector<ActionJob>& jobs, const std::vector<Csr
   int want = 1;
   while (want < 16 && want * 64 < S.dmax) want *= 2;
   S.cap = 0;
-  S.cluster = want > 1 ? action_cluster_size(want, S.dmax, 0) : 1;
+  const int regs = longest <= 8 ? 8 : longest <= 16 ? 16 : 24;
+  S.cluster = want > 1 ? action_rows_cluster_size(want, S.dmax, regs) : 1;
   if ((S.dmax + S.cluster - 1) / S.cluster > 256) return false;
-  S.row_regs = longest <= 8 ? 8 : longest <= 16 ? 16 : 24;
+  S.row_regs = regs;
   return true;
 }
 // A few large jobs run as one thread block cluster each (up to 16 CTAs, about

@@ -264,6 +264,7 @@ size_t action_smem_bytes(int dmax, int nnz_cap);
 size_t action_cluster_smem_bytes(int dmax, int C, int cap_loc);
 // largest power-of-two cluster size <= want that the device co-schedules, else 1
 int action_cluster_size(int want, int dmax, int cap_loc);
+int action_rows_cluster_size(int want, int dmax, int row_regs);   // of the real-row kernel
 // bounds kernel, then the chain: one CTA per job (cluster <= 1, nnz_cap = the
 // nonzeros held on chip) or one cluster of `cluster` CTAs per job (nnz_cap =
 // own-row nonzeros held on chip per CTA)
