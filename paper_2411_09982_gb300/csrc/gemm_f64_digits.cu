@@ -63,6 +63,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 
 namespace mg {
 
@@ -100,16 +101,20 @@ static F8Geom f8_geom(int d) {
   return g;
 }
 
-// The product's kernels have to be compiled to the register count their split starts from.
-static int f8_check_registers(const void* kern) {
+// The product's kernels have to be compiled to the register count their split starts from
+// (asked for once per kernel).
+static int f8_check_registers(const void* kern, std::atomic<bool>& checked) {
+  if (checked.load(std::memory_order_relaxed)) return MG_OK;
   cudaFuncAttributes at;
   MG_CUDA_TRY(cudaFuncGetAttributes(&at, kern));
   if (at.numRegs < F8_REGS_LAUNCH) {
     set_last_message("the FP64 digit product is compiled to %d registers, its split needs %d", at.numRegs, F8_REGS_LAUNCH);
     return MG_EUNSUPPORTED;
   }
+  checked.store(true, std::memory_order_relaxed);
   return MG_OK;
 }
+static std::atomic<bool> f8_checked[2];
 
 // operand buffer: digits of all items, then row (column) exponents, then the items' marks and
 // digit energies
@@ -1230,7 +1235,7 @@ int f64d_gemm(int d, int batch, int opA, const double* A, long long sA, const vo
   const int grid = (int)std::min<long long>(std::max(tiles, (sub * sub * batch + 1) / 2), sms);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<true>), (int)smem));
-  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<true>)));
+  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<true>), f8_checked[0]));
   f64d_gemm_kernel<true><<<grid, F8_THREADS, smem, s>>>(ma, mb, p);
   MG_TRY(check_launch("f64d_gemm_kernel"));
   return MG_OK;
@@ -1282,7 +1287,7 @@ int f64r_expm(int d, int batch, const double* W, const double* tau, int m, int s
   const int ntm = ceil_div(d, F8_BM);
   const size_t smem = (size_t)F8_SLOTS * F8_SLOT_BYTES + F8_STAGE_BYTES + 256 + 1024;
   MG_TRY(ensure_smem_limit(reinterpret_cast<const void*>(f64d_gemm_kernel<false>), (int)smem));
-  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<false>)));
+  MG_TRY(f8_check_registers(reinterpret_cast<const void*>(f64d_gemm_kernel<false>), f8_checked[1]));
   // dst = 2^scale2 D[x] D[y] + sum_m coef_m src_m + diag I
   auto mul = [&](int x, int y, double* dst, int n, const double* const* src, const double* coef, double diag,
                  int scale2) {
