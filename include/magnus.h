@@ -70,6 +70,9 @@ extern "C" {
  *   d 2^-53 sum_k |a_ik| |b_kj|: 128 x 64 blocks with weaker entries than the digits hold so
  *   take native FP64 arithmetic, 2 to 20 times slower.  So do operands with a NaN, an
  *   infinity or a row or column scale outside 2^-400 .. 2^400, small products and mg_cgemm.
+ *   Which products are small follows from d and the batch, so the last bits of a result
+ *   depend on how a call is cut: on N, the workspace limit and the other jobs of a batch, as
+ *   the Taylor degree of a chunk does.
  *   If a bounded device wait of a product on the tensor cores gives up, its outputs become
  *   NaN and the next call that reads the context's status returns MG_ETIMEOUT (the same call
  *   when it reports or copies to the host).

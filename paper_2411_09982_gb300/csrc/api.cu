@@ -359,9 +359,16 @@ int timing_mark(mg_ctx* ctx, int* idx) {
 // FP64 products run from digits on the tensor cores (gemm_f64_digits.cu) from d = 33 on and
 // where the batch is worth it: from digits a small batch costs its slicers and one wave of
 // tiles however little work it is, on the FP64 pipe its work.  The two meet at dp^3 batch =
-// 6e6 to 1e7 (dp: d rounded up to the pipe kernel's 16-wide tiles) at every d; exponentials
-// from digits / on the pipe: one of d = 100 820 / 435 us, one of d = 200 1085 / 1200, 16 of
-// d = 64 600 / 449, 32 609 / 749, 128 751 / 2263, 8 of d = 128 882 / 1480.
+// 6e6 to 1e7 (dp: d rounded up to the pipe kernel's 16-wide tiles) for exponentials of either
+// form and for single products alike.  A call of one chunk, digits / pipe in us, norm 3:
+//   real symmetric exponentials: 64 of d = 40 (7.1e6) 713 / 660, 128 893 / 1133; 16 of d = 64
+//   (4.2e6) 605 / 481, 32 666 / 784; 4 of d = 100 (5.6e6) 696 / 597, 8 734 / 843; 2 of d = 128
+//   (4.2e6) 682 / 448, 4 706 / 720, 8 744 / 1284; one of d = 200 (9e6) 889 / 1055;
+//   complex ones: the same pipe times, digits 702, 886; 612, 655; 721, 757; 722, 751, 801; 951;
+//   one level of a tree: 32 products of d = 64 (8.4e6) 64 / 71, 8 of d = 100 (1.1e7) 82 / 82,
+//   4 of d = 128 (8.4e6) 81 / 74, 8 84 / 133, one of d = 200 (9e6) 122 / 128 with its call.
+// So the bits of an interval's U_n depend on what shares its chunk, as its degree and squaring
+// count do.
 constexpr int kF64DigitsMinDim = 33;
 bool f64_digits_pay(int d, int batch) {
   const long long dp = (d + 15) / 16 * 16;
