@@ -380,6 +380,7 @@ struct Engine {
   int d, prec, L;
   void* abuf = nullptr;
   void* bbuf[2] = {nullptr, nullptr};
+  int reserved = 0;                   // largest batch the operand slots were asked for
   long long products = 0;
   // split products: with item_sq set, only items with item_sq[b] > sq_step are sliced and
   // multiplied (per-interval squaring counts; see expm_chunk_dev)
@@ -420,6 +421,7 @@ struct Engine {
   }
 
   int reserve(int batch) {
+    reserved = std::max(reserved, batch);
     if (digits64(batch)) {
       MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(d, batch), &abuf));
       MG_TRY(ws_get(ctx, WS_BBUF0, f64d_b_bytes(d, batch), &bbuf[0]));
@@ -889,17 +891,19 @@ int expm_chunk_dev(mg_ctx* ctx, Engine& eng, int batch, double* W, const double*
 
 // C = opA(A) B in FP64 (report and re-orthonormalisation products): from digits where the
 // engine's FP64 products are, else on the FP64 pipe.  Uses the operand slots of `eng`, as many
-// items at a time as those hold (split precision with few slices reserves less than FP64
-// digits take).  Entry by entry only where the engine's products are FP64 ones (split states
+// items at a time as its own reservation holds (split precision with few slices reserves less
+// than FP64 digits take).  What the slots hold from elsewhere does not count: a captured run
+// must take the launches and sizes of the run before it.  Entry by entry only where the engine's products are FP64 ones (split states
 // carry larger errors, and the report takes the largest entry of its product).
 int mul_f64(mg_ctx* ctx, Engine& eng, int batch, int opA, const double* A, const double* B, double* C) {
   const long long md = mat_doubles(eng.d);
   AddTerms none;
   Engine e{ctx, eng.d, MG_PREC_FP64, 0};
   int nb = batch;
-  if (e.digits_dim() && eng.abuf && eng.bbuf[0])
-    nb = (int)std::min<size_t>(nb, std::max<size_t>(1, std::min(ctx->slot_size[WS_ABUF] / f64d_a_bytes(e.d, 1),
-                                                                ctx->slot_size[WS_BBUF0] / f64d_b_bytes(e.d, 1))));
+  if (eng.df() && eng.reserved > 0)
+    nb = (int)std::min<size_t>(nb, std::max<size_t>(1, std::min(
+             split_a_bytes(eng.d, eng.L, eng.reserved) / f64d_a_bytes(e.d, 1),
+             split_b_bytes(eng.d, eng.L, eng.reserved) / f64d_b_bytes(e.d, 1))));
   if (!e.digits64(nb)) return launch_cgemm_f64(batch, e.d, A, md, opA, B, md, C, md, none, ctx->stream);
   void *ab, *bb, *sums;
   MG_TRY(ws_get(ctx, WS_ABUF, f64d_a_bytes(e.d, nb), &ab));

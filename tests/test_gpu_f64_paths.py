@@ -179,3 +179,33 @@ def test_fp64_chunks_without_digits_are_not_cut_for_them():
         plan.close()
         ctx.close()
     assert launches[0] == launches[1]
+
+
+def test_captured_batch_takes_the_products_of_the_run_before_it():
+    """Re-orthonormalised propagators of d = 64 beside states of d = 128, two slices: by the time
+    of the capture the second group has grown the operand slots, which must not change the first
+    group's FP64 products (how many at a time, and so whether from digits)."""
+    rng = np.random.default_rng(4)
+    ctx = M.Context(0, stream=torch.cuda.Stream())   # the default stream cannot be captured
+    try:
+        plans, outs, ins, kinds = [], [], [], []
+        for d, N, kind in ((64, 70, M.MG_OUT_PROPAGATOR), (128, 200, M.MG_OUT_STATE)):
+            p = M.Plan(ctx, cuda(hermitian(rng, d, 0.5, False)), None, M.MG_PREC_SPLIT, 2)
+            p.set_controls(N, 1, 0.0, 1.0, np.array([2.0]), torch.zeros((N, 1, 0), dtype=torch.float64))
+            plans.append(p)
+            kinds.append(kind)
+            shape = (d, d) if kind == M.MG_OUT_PROPAGATOR else (d,)
+            outs.append(torch.empty(shape, dtype=torch.complex128, device="cuda"))
+            ins.append(None if kind == M.MG_OUT_PROPAGATOR else cuda(np.eye(d)[0].astype(np.complex128)))
+        torch.cuda.synchronize()
+        g = M.BatchGraph(ctx, plans, kinds, ins, outs, 2)
+        g.launch()
+        torch.cuda.synchronize()
+        got = [o.clone() for o in outs]
+        g.close()
+        assert M.mg_evolve_batch(ctx, plans, kinds, ins, outs, 2) == [0, 0]
+        torch.cuda.synchronize()
+        for a, b in zip(got, outs):
+            assert torch.equal(a, b)
+    finally:
+        ctx.close()
