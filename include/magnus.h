@@ -618,7 +618,7 @@ int mg_ctx_set_structure(mg_ctx* ctx, int on);
 /* MG_PREC_FP64 entry by entry: on != 0 runs every FP64 product of the context's calls in native
  * FP64 arithmetic, also those that digits would give (evolutions, batches, servers; the
  * products of re-orthonormalisation and of the report in either precision), so that weak
- * amplitudes keep 53 bits of their own.  One product of d = 729: 2.6 ms instead of 0.1.
+ * amplitudes keep 53 bits of their own.  One product of d = 729: 2.5 ms instead of 0.1.
  * 0 (the default) as described at MG_PREC_FP64. */
 int mg_ctx_set_fp64_entrywise(mg_ctx* ctx, int on);
 int mg_ctx_gemm_stats(mg_ctx* ctx, int64_t* launches, double* ms, double* flops, int reset);

@@ -48,9 +48,10 @@
 //               while levels 0..3 are swept onto the high ones.  Rounding to FP64, addends
 //               and stores run while the next tile's MMAs are issued.  These warps take
 //               registers over from the first four (setmaxnreg).
-// Measured (GB300, one product of a batch, slicing included): d = 729 2804 us on the FP64
-// pipe -> 106 us (29 TFLOP/s of the product's 8 d^3); d = 256 112 -> 7.6 us; d = 81 8.9 ->
-// 1.2 us.  Small K is bound by the epilogue's latency, which is why it has 16 warps (eight
+// Measured (GB300, one product of a batch, slicing included, against the FP64-pipe kernel of
+// gemm_f64.cu): d = 729, batch 16 2531 -> 103 us (30 TFLOP/s of the product's 8 d^3); d = 256,
+// batch 128 108 -> 5.4 us; d = 81, batch 256 5.0 -> 0.86 us.  The tensor pipe is 55% busy at
+// d = 256 and 729, 29% at d = 81.  Small K is bound by the epilogue's latency, which is why it has 16 warps (eight
 // warps of 64 sums: d = 84 exponentials 2.93 -> 2.42 ms, d = 256 12.1 -> 10.7, d = 729 the
 // same); at d = 729 the slicers take 12% (HBM-bound), the drains 11%, and the operands arrive
 // at 43 bytes per cycle and SM, near what L2 delivers.
