@@ -815,8 +815,8 @@ int expm_chunk(mg_ctx* ctx, Engine& eng, int batch, double* W, const double* tau
   // itself has weak entries beside a diagonal of ones where X is small (a batch of norms 0.1 to
   // 20 squares all of its items as often as the largest), which the digits do not hold to
   // FP64's bound: 64 dense matrices of d = 81 took FP64 arithmetic in many tiles, 3.9 ms
-  // against 1.5 on E, whose entries are of one size.  (1.2 without the check of the products;
-  // relative error 9e-15 unchecked on T, 2.9e-15 so.)
+  // against 1.4 on E, whose entries are of one size.  (1.2 without the check of the products;
+  // relative error 9e-15 unchecked on T, 2.7e-15 so.)
   const bool less_identity = eng.entrywise && eng.digits64(batch);
   MG_TRY(taylor_poly(ctx, eng, batch, W, tc, &R, &Rn, less_identity));
   // squarings

@@ -475,8 +475,11 @@ __device__ __forceinline__ bool f8_skip(const F8Args& p, int b, long long t) {
 // rounded down, scaled by 2^{57 - Ea}, 2^{57 - Eb}) and sends a tile to FP64 arithmetic where
 // an entry has M + |P| / d < 2^{114 - 8} / sqrt(d).  M = 0 is a zero of the operands'
 // structure, which the digits give exactly, unless some entry in reach is below 2^-110 of its
-// row or column.  128 x 64 outputs per CTA (the product's tiles), 4 x 4 per thread; small d is
-// bound by latency: d = 81, batch 64 takes 16 us a product (256 threads of 8 x 4 outputs: 42).
+// row or column.  128 x 64 outputs per CTA (the product's tiles), 4 x 4 per thread, K in slabs of
+// 16 until every output of the tile holds: the terms only add up.  Bound by latency.  Exponentials
+// of dense matrices, in us without the check / with every K / as it is: 64 of d = 64 1012 / 1218 /
+// 1149, 37 of d = 100 1294 / 1582 / 1438, 10 of d = 200 1632 / 2080 / 1767, 5 of d = 400 2268 /
+// 3029 / 2424.  (256 threads of 8 x 4 outputs took 42 us a launch at d = 81, batch 64, against 16.)
 constexpr int F8_NK = 16;              // K per slab
 constexpr int F8_WEAK_THREADS = 512;
 // the larger component's magnitude times 2^k, rounded down (0 below FP32's normal range,
@@ -530,8 +533,19 @@ f64d_weak_kernel(const __grid_constant__ F8Args p, float least, unsigned char* _
   for (int q = 0; q < 4; ++q) Ea[q] = i0 + row(q) < d ? f8_exponent(ea[i0 + row(q)]) : 0;
   const int c0 = (tid & 15) * 4, r0 = (tid >> 4) * 4;   // outputs: 4 x 4
   constexpr float kTiny = 1.1102230246251565e-16f;      // 2^{57 - 110}
-  float m[4][4] = {};
+  const float per_d = 1.0f / (float)d;
+  float m[4][4] = {}, add[4][4] = {};                   // M so far, |P| / d
   bool tiny = false;
+  // an output of this thread does not hold the bound with the terms so far (zero: M = 0 counts)
+  auto short_of = [&](bool zero) {
+    bool low = false;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        low |= i0 + r0 + r < d && j0 + c0 + c < d && m[r][c] + add[r][c] < least && (m[r][c] > 0.f || zero);
+    return low;
+  };
   for (int k0 = 0; k0 < d; k0 += F8_NK) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -558,28 +572,32 @@ f64d_weak_kernel(const __grid_constant__ F8Args p, float least, unsigned char* _
           for (int c = 0; c < 4; ++c) m[r][c] = fmaf(xs[r], ys[c], m[r][c]);
       }
     }
-    __syncthreads();
+    // M only grows: a tile of dense operands is done after one slab, with addends after two
+    if (!__syncthreads_or(short_of(true))) {
+      if (tid == 0) weak[t] = 0;
+      return;
+    }
+    if (k0 == 0) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int i = i0 + r0 + r, j = j0 + c0 + c;
+          if (i >= d || j >= d) continue;
+          const int k = 114 - f8_exponent(ea[i]) - f8_exponent(eb[j]);
+          float v = i == j ? f8_magnitude(make_double2(p.diag, 0.0), k) : 0.f;
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+            if (q < p.add_n) {
+              const float x = f8_magnitude(reinterpret_cast<const double2*>(p.add_src[q] + b * p.add_stride)[(long long)i * d + j], k);
+              if (x > 0.f) v = fmaf(fabsf((float)p.add_coef[q]), x, v);
+            }
+          add[r][c] = v * per_d;
+        }
+    }
   }
   const bool any_tiny = __syncthreads_or(tiny);
-  const float per_d = 1.0f / (float)d;
-  bool low = false;
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int i = i0 + r0 + r, j = j0 + c0 + c;
-      if (i >= d || j >= d || m[r][c] >= least || (m[r][c] == 0.f && !any_tiny)) continue;
-      const int k = 114 - f8_exponent(ea[i]) - f8_exponent(eb[j]);
-      float add = i == j ? f8_magnitude(make_double2(p.diag, 0.0), k) : 0.f;
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (q < p.add_n) {
-          const float x = f8_magnitude(reinterpret_cast<const double2*>(p.add_src[q] + b * p.add_stride)[(long long)i * d + j], k);
-          if (x > 0.f) add = fmaf(fabsf((float)p.add_coef[q]), x, add);
-        }
-      low |= !(m[r][c] + add * per_d >= least);
-    }
-  low = __syncthreads_or(low);
+  const bool low = __syncthreads_or(short_of(any_tiny));
   if (tid == 0) weak[t] = low;
 }
 
