@@ -46,6 +46,32 @@ def test_shear_squared(d):
         ctx.close()
 
 
+@pytest.mark.parametrize("width", [0.5, 2.0, 6.0, 20.0, 1e9])
+@pytest.mark.parametrize("d", [33, 65, 129, 300])
+def test_graded_operands_hold_the_bound(d, width):
+    """Entries falling by 2^-(distance from the diagonal / width): tiles on either side of the
+    check's line.  FP64 arithmetic keeps (2 d + 2) u M, M = |A| |B|; tiles from digits pass the
+    check with a standard error below d u M, taken eightfold."""
+    rng = np.random.default_rng(d)
+    ctx = M.Context(0)
+    try:
+        fall = 2.0 ** -(np.abs(np.subtract.outer(np.arange(d), np.arange(d))) / width)
+        A, B = ((rng.normal(size=(d, d)) + 1j * rng.normal(size=(d, d))) * fall for _ in range(2))
+        n = enough(d)
+        U = torch.eye(d, dtype=torch.complex128, device="cuda").repeat(2 * n, 1, 1)
+        U[0], U[1] = cuda(B), cuda(A)
+        out = torch.empty((d, d), dtype=torch.complex128, device="cuda")
+        M.mg_propagate(ctx, 2 * n, d, U, M.MG_OUT_PROPAGATOR, None, out, 0, M.MG_PREC_FP64)
+        C = out.cpu().numpy()
+        rows = np.unique(np.linspace(0, d - 1, 40).astype(int))
+        Ar, Ai, Br, Bi = (x.astype(np.longdouble) for x in (A.real[rows], A.imag[rows], B.real, B.imag))
+        bound = 8 * d * 2.0 ** -53 * (np.abs(A[rows]) @ np.abs(B))
+        assert np.all(np.abs((C.real[rows] - (Ar @ Br - Ai @ Bi)).astype(np.float64)) <= bound)
+        assert np.all(np.abs((C.imag[rows] - (Ar @ Bi + Ai @ Br)).astype(np.float64)) <= bound)
+    finally:
+        ctx.close()
+
+
 def expm_dense(T):
     """exp(T) by scaling and squaring of the Taylor series, entries of one size."""
     s = max(0, int(np.ceil(np.log2(np.abs(T).sum(0).max()))) + 3)
